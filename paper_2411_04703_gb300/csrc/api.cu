@@ -902,7 +902,7 @@ int step_once(pic_ctx *c)
     if (sorted) {
         TraceScope ts(c, TR_SORT);
         for (int si = 0; si < c->nsp; si++)
-            if (!c->sp[si].lattice) CK(launch_sort(c, si));
+            if (!c->sp[si].lattice) CK(launch_sort(c, si, !c->sp[si].frozen));
     }
     if (c->ad_rec_n >= 0) {
         if (c->ad_rec_n >= (int)c->ad_rec.size()) return fail(c, PIC_ERR_STATE, "adjoint record overflow");
@@ -1464,7 +1464,7 @@ int pic_sort(pic_ctx *c)
     if (r) return r;
     TraceScope ts(c, TR_SORT);
     for (int si = 0; si < c->nsp; si++)
-        if (!c->sp[si].lattice) CK(launch_sort(c, si));
+        if (!c->sp[si].lattice) CK(launch_sort(c, si, false));
     return PIC_OK;
 }
 

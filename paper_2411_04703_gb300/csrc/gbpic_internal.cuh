@@ -136,7 +136,7 @@ struct TileDev {
     const int *cell_start;   // [n_keys + 1]: first sorted slot of each key (8 keys per cell), valid
                              // for the tiles holding particles at the last sort
     const int *tile_start;   // [ntiles + 1]: first sorted slot of each tile (the last: the live count)
-    const int2 *items;       // (tile, chunk) work items of the tiles with >= kSparse particles
+    const int4 *items;       // work items of the tiles with >= kSparse particles: tile, first slot, end slot
     const int *sparse_tiles; // tiles with 1 .. kSparse-1 particles (count[3] of them)
     int chunk;               // particles per work item (kChunkMin .. kChunk), fixed at the sort
     CellCode cc;
@@ -176,7 +176,7 @@ struct Species {
     int *id = nullptr, *id2 = nullptr;
     int *count = nullptr;     // device [4]
     int *rank = nullptr;      // device [cap] sort scratch
-    int2 *items = nullptr;    // device work items
+    int4 *items = nullptr;    // device work items
     int64_t max_items = 0;
     int *cell_start = nullptr;  // device [n_keys + 1]; zero outside the tiles listed in occ
     int *tile_start = nullptr;  // device [ntiles + 1]: particles per tile, then their exclusive scan
@@ -343,7 +343,7 @@ cudaError_t launch_snap_arm(pic_ctx *c);
 cudaError_t launch_snap_record(pic_ctx *c);
 cudaError_t launch_snap_moments(pic_ctx *c, double k, double *out);
 // k_sort.cu
-cudaError_t launch_sort(pic_ctx *c, int si);
+cudaError_t launch_sort(pic_ctx *c, int si, bool by_octant);
 cudaError_t exclusive_scan(pic_ctx *c, int *data, int64_t n);
 int64_t scan_scratch_size(int64_t n);
 // k_init.cu

@@ -1,17 +1,19 @@
-// The dispatcher over the particle kernel's variants (shape order, frozen or mobile, region
-// shape; the second-order variants are compiled in k_push2_*.cu, the first-order ones in
-// k_push1.cu) and the charge-density deposit used by pic_get_fields(RHO).
+// The dispatcher over the particle kernels' variants (shape order, frozen or mobile, gather scheme,
+// region shape), each compiled in a translation unit of its own (k_push1*.cu, k_push2_*.cu), and the charge-density deposit used by pic_get_fields(RHO).
 #include "push_impl.cuh"
 
 namespace gbpic {
 
-cudaError_t launch_push_order1(pic_ctx *c, int si, const ExtDev &ext);
-cudaError_t launch_push2_mobile_fixed(pic_ctx *c, int si, const ExtDev &ext);
-cudaError_t launch_push2_frozen_fixed(pic_ctx *c, int si, const ExtDev &ext);
-cudaError_t launch_push2_mobile_dyn(pic_ctx *c, int si, const ExtDev &ext);
-cudaError_t launch_push2_frozen_dyn(pic_ctx *c, int si, const ExtDev &ext);
-cudaError_t launch_push2_mobile_fixed_ec(pic_ctx *c, int si, const ExtDev &ext);
-cudaError_t launch_push2_mobile_dyn_ec(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push1_frozen(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push1_fixed(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push1_fixed_ec(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push1_dyn(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push1_dyn_ec(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push2_frozen(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push2_fixed(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push2_fixed_ec(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push2_dyn(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push2_dyn_ec(pic_ctx *c, int si, const ExtDev &ext);
 
 namespace {
 
@@ -96,15 +98,15 @@ cudaError_t launch_dlim_from_momenta(pic_ctx *c, int si)
 
 cudaError_t launch_push(pic_ctx *c, int si, const ExtDev &ext)
 {
-    if (c->order == 1) return launch_push_order1(c, si, ext);
-    const bool fr = c->sp[si].frozen != 0;
+    const bool o1 = c->order == 1;
+    if (c->sp[si].frozen) return o1 ? launch_push1_frozen(c, si, ext) : launch_push2_frozen(c, si, ext);
     const bool ec = c->gather == PIC_GATHER_ENERGY;
     if (push::default_region(c)) {
-        if (fr) return launch_push2_frozen_fixed(c, si, ext);
-        return ec ? launch_push2_mobile_fixed_ec(c, si, ext) : launch_push2_mobile_fixed(c, si, ext);
+        if (o1) return ec ? launch_push1_fixed_ec(c, si, ext) : launch_push1_fixed(c, si, ext);
+        return ec ? launch_push2_fixed_ec(c, si, ext) : launch_push2_fixed(c, si, ext);
     }
-    if (fr) return launch_push2_frozen_dyn(c, si, ext);
-    return ec ? launch_push2_mobile_dyn_ec(c, si, ext) : launch_push2_mobile_dyn(c, si, ext);
+    if (o1) return ec ? launch_push1_dyn_ec(c, si, ext) : launch_push1_dyn(c, si, ext);
+    return ec ? launch_push2_dyn_ec(c, si, ext) : launch_push2_dyn(c, si, ext);
 }
 
 // Adds the charge density of species s to rho.

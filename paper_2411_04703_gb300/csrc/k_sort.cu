@@ -13,23 +13,26 @@ constexpr int kScanThreads = 1024;
 constexpr int kScanSeg = 2 * kScanThreads;
 
 // Sort key of a particle: tiles in x-fastest order; inside a tile the cells in (x fastest, z,
-// y) order; inside a cell the octant of the offset (bit d set when offset_d >= 1/2).  A warp's
-// 32 consecutive cells then form an 8 x 4 (x, z) block at one y, and the particles of a cold
-// lattice come in the same octant order in every cell.
-__device__ __forceinline__ int tile_key(const float4 &P, const TileDev &t)
+// y) order; inside a cell the octant of the offset (bit d set when offset_d >= 1/2).
+// by_octant (the steps of mobile species): inside a tile the cells of one y row, then the octant,
+// then z, then x: 32 consecutive particles of a lattice with up to two particles a cell and dim are
+// then on 32 cells of an 8 x 4 (x, z) block at the same place in their cells, so that a warp of the
+// particle kernel reads and writes whole lines of records and meets no bank twice.
+__device__ __forceinline__ int tile_key(const float4 &P, const TileDev &t, bool by_octant)
 {
     const int cell = __float_as_int(P.w);
     const int i = t.cc.i(cell), j = t.cc.j(cell), k = t.cc.k(cell);
     const int tile = ((k / t.T[2]) * t.nt[1] + j / t.T[1]) * t.nt[0] + i / t.T[0];
-    const int local = ((j % t.T[1]) * t.T[2] + k % t.T[2]) * t.T[0] + i % t.T[0];
+    const int lx = i % t.T[0], ly = j % t.T[1], lz = k % t.T[2];
     const int oct = (P.x >= 0.5f) | ((P.y >= 0.5f) << 1) | ((P.z >= 0.5f) << 2);
-    return (tile * t.tile_cells + local) * 8 + oct;
+    const int local = by_octant ? ((ly * 8 + oct) * t.T[2] + lz) * t.T[0] + lx : ((ly * t.T[2] + lz) * t.T[0] + lx) * 8 + oct;
+    return tile * t.tile_cells * 8 + local;
 }
 
 // Key counters (the rank of each particle among its key) and particles per tile.  The lanes of a
 // warp mostly share a tile (the particles were sorted by tile last time), so a tile's counter
 // takes one atomic per warp.
-__global__ void k_sort_count(SpeciesDev sp, TileDev t, int n_keys, int *hist, int *rank, int *tile_cnt)
+__global__ void k_sort_count(SpeciesDev sp, TileDev t, bool by_octant, int n_keys, int *hist, int *rank, int *tile_cnt)
 {
     const int n = sp.count[0];
     const int kpt = t.tile_cells * 8;
@@ -40,7 +43,7 @@ __global__ void k_sort_count(SpeciesDev sp, TileDev t, int n_keys, int *hist, in
         if (p < n) {
             const float4 P = sp.pos[p];
             const bool live = __float_as_int(P.w) >= 0;
-            const int key = live ? tile_key(P, t) : n_keys;
+            const int key = live ? tile_key(P, t, by_octant) : n_keys;
             rank[p] = atomicAdd(hist + key, 1);
             if (live) tile = key / kpt;
         }
@@ -137,7 +140,7 @@ __global__ void __launch_bounds__(kTileScanThreads) k_tile_scan(int *hist, const
     }
 }
 
-__global__ void k_sort_scatter(SpeciesDev sp, TileDev t, int n_keys, const int *start, const int *rank,
+__global__ void k_sort_scatter(SpeciesDev sp, TileDev t, bool by_octant, const int *start, const int *rank,
                                float4 *pos2, float4 *mom2, int *id2)
 {
     const int n = sp.count[0];
@@ -145,7 +148,7 @@ __global__ void k_sort_scatter(SpeciesDev sp, TileDev t, int n_keys, const int *
         const float4 P = sp.pos[p];
         const int cell = __float_as_int(P.w);
         if (cell < 0) continue;
-        const int dst = start[tile_key(P, t)] + rank[p];
+        const int dst = start[tile_key(P, t, by_octant)] + rank[p];
         pos2[dst] = P;
         mom2[dst] = sp.mom[p];
         id2[dst] = sp.id[p];
@@ -169,13 +172,14 @@ __global__ void k_tile_chunks(const int *tile_start, int ntiles, int chunk, int 
     sparse_flag[tl] = sparse ? 1 : 0;
 }
 
-__global__ void k_fill_items(const int *chunk_start, const int *sparse_start, int ntiles, int2 *items,
+__global__ void k_fill_items(const int *chunk_start, const int *sparse_start, int ntiles, int chunk, int4 *items,
                              int *sparse_tiles, int *count, const int *tile_start)
 {
     const int tl = blockIdx.x * blockDim.x + threadIdx.x;
     if (tl < ntiles) {
         const int b = chunk_start[tl], e = chunk_start[tl + 1];
-        for (int c = b; c < e; c++) items[c] = make_int2(tl, c - b);
+        const int p0 = tile_start[tl], p1 = tile_start[tl + 1];
+        for (int c = b; c < e; c++) items[c] = make_int4(tl, p0 + (c - b) * chunk, min(p0 + (c - b + 1) * chunk, p1), 0);
         if (sparse_start[tl + 1] > sparse_start[tl]) sparse_tiles[sparse_start[tl]] = tl;
     }
     if (tl == 0) {
@@ -265,7 +269,7 @@ cudaError_t exclusive_scan(pic_ctx *c, int *data, int64_t n)
     return scan_rec(c->stream, data, n, c->hist_tmp, c->kernels);
 }
 
-cudaError_t launch_sort(pic_ctx *c, int si)
+cudaError_t launch_sort(pic_ctx *c, int si, bool by_octant)
 {
     Species &s = c->sp[si];
     // work items small enough that a small species still gives every SM one (each item stages a
@@ -284,21 +288,21 @@ cudaError_t launch_sort(pic_ctx *c, int si)
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(s.occ + c->ntiles, 0, sizeof(int), c->stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(s.tile_start, 0, sizeof(int) * (c->ntiles + 1), c->stream)) != cudaSuccess) return e;
-    k_sort_count<<<grid, 256, 0, c->stream>>>(sd, t, n_keys, s.cell_start, s.rank, s.tile_start);
+    k_sort_count<<<grid, 256, 0, c->stream>>>(sd, t, by_octant, n_keys, s.cell_start, s.rank, s.tile_start);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = exclusive_scan(c, s.tile_start, c->ntiles + 1)) != cudaSuccess) return e;
     k_occ_list<<<(c->ntiles + 255) / 256, 256, 0, c->stream>>>(s.tile_start, c->ntiles, s.occ);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_tile_scan<<<c->num_sms * 4, kTileScanThreads, 0, c->stream>>>(s.cell_start, s.tile_start, s.occ, c->ntiles, kpt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_sort_scatter<<<grid, 256, 0, c->stream>>>(sd, t, n_keys, s.cell_start, s.rank, s.pos2, s.mom2, s.id2);
+    k_sort_scatter<<<grid, 256, 0, c->stream>>>(sd, t, by_octant, s.cell_start, s.rank, s.pos2, s.mom2, s.id2);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_tile_chunks<<<(c->ntiles + 1 + 255) / 256, 256, 0, c->stream>>>(s.tile_start, c->ntiles, s.chunk, s.chunk_start,
                                                                        s.sparse_start);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = exclusive_scan(c, s.chunk_start, c->ntiles + 1)) != cudaSuccess) return e;
     if ((e = exclusive_scan(c, s.sparse_start, c->ntiles + 1)) != cudaSuccess) return e;
-    k_fill_items<<<(c->ntiles + 255) / 256, 256, 0, c->stream>>>(s.chunk_start, s.sparse_start, c->ntiles, s.items,
+    k_fill_items<<<(c->ntiles + 255) / 256, 256, 0, c->stream>>>(s.chunk_start, s.sparse_start, c->ntiles, s.chunk, s.items,
                                                                   s.sparse_tiles, s.count, s.tile_start);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     c->kernels += 7;   // zero, count, occupied list, tile scan, scatter, tile_chunks, fill_items

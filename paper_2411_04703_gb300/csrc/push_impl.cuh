@@ -45,11 +45,11 @@ struct RegDyn {
     __device__ __forceinline__ int r2() const { return R2; }
     __device__ __forceinline__ int r3() const { return R3; }
 };
-template <int RX, int RY, int RZ> struct RegFix {
+template <int RX, int RY, int RZ, int R2 = plane_pitch(RX, RY)> struct RegFix {
     __device__ __forceinline__ static constexpr int rx() { return RX; }
     __device__ __forceinline__ static constexpr int ry() { return RY; }
-    __device__ __forceinline__ static constexpr int r2() { return plane_pitch(RX, RY); }
-    __device__ __forceinline__ static constexpr int r3() { return plane_pitch(RX, RY) * RZ; }
+    __device__ __forceinline__ static constexpr int r2() { return R2; }
+    __device__ __forceinline__ static constexpr int r3() { return R2 * RZ; }
 };
 
 // ------------------------------------------------------------------ shape weights
@@ -208,6 +208,9 @@ template <class Reg> struct SmemAcc {
     // v is already in fixed-point units (times scale(comp)), |v| <= 2^30
     __device__ __forceinline__ void j(int comp, const int st[3], int i, int j, int k, float v) const {
         const int ix = comp * reg.r3() + base + (st[2] + k) * reg.r2() + (st[1] + j) * reg.rx() + st[0] + i;
+        add(ix, v);
+    }
+    __device__ __forceinline__ void add(int ix, float v) const {
         const int V = __float2int_rn(v);
         atomicAdd(&sJlo[ix], (unsigned)V & kLoMask);
         atomicAdd(&sJhi[ix], V >> kLoBits);
@@ -399,29 +402,10 @@ __device__ __forceinline__ void deposit_simple(Acc &acc, const float o[3], const
     esirkepov<L, false>(acc, st, S0, DS, fac, d[0] == 0.f, d[1] == 0.f);
 }
 
-// Gather, external field and Boris rotation of one particle: u^{n-1/2} -> u^{n+1/2} in mo.
-// GATHER 0: momentum-conserving (the deposit's shape at each component's Yee point); GATHER 1:
-// energy-conserving (one order lower along the component's staggered dims: the transpose of the
-// Esirkepov deposit, whose J_x has the lower-order shape at the half-integer x nodes).
-template <int ORDER, class Acc, int GATHER = 0>
-__device__ __forceinline__ void push_u(Acc &acc, const float o[3], const int c[3], float4 &mo,
-                                       const SpeciesDev &sp, const ExtDev &ext)
+// External field and momentum push of one particle in the gathered E, B: u^{n-1/2} -> u^{n+1/2} in mo.
+__device__ __forceinline__ void kick(const float o[3], const int c[3], float E[3], float B[3], float4 &mo,
+                                     const SpeciesDev &sp, const ExtDev &ext)
 {
-    using S = Shape<ORDER>;
-    using SS = Shape<GATHER ? ORDER - 1 : ORDER>;   // shape along staggered dims
-    constexpr int N = S::N, NS = SS::N;
-    int su[3], ss[3];
-    float wu[3][N], ws[3][NS];
-#pragma unroll
-    for (int dd = 0; dd < 3; dd++) { S::unst(o[dd], su[dd], wu[dd]); SS::stag(o[dd], ss[dd], ws[dd]); }
-    float E[3], B[3];
-    acc.template gather_windows<N, NS>(su, ss);
-    E[0] = gather3<true, false, false, N, NS>(acc, 0, su, ss, wu, ws);
-    E[1] = gather3<false, true, false, N, NS>(acc, 1, su, ss, wu, ws);
-    E[2] = gather3<false, false, true, N, NS>(acc, 2, su, ss, wu, ws);
-    B[0] = gather3<false, true, true, N, NS>(acc, 3, su, ss, wu, ws);
-    B[1] = gather3<true, false, true, N, NS>(acc, 4, su, ss, wu, ws);
-    B[2] = gather3<true, true, false, N, NS>(acc, 5, su, ss, wu, ws);
     if (ext.type == PIC_EXT_PLANAR_UNDULATOR || ext.type == PIC_EXT_PLANAR_UNDULATOR_3D) {
         float f = 1.f;
         if (ext.ramp_mode) {
@@ -482,23 +466,50 @@ __device__ __forceinline__ void push_u(Acc &acc, const float o[3], const int c[3
     mo.z = um[2] + up[0] * sv[1] - up[1] * sv[0] + h * E[2];
 }
 
-// Gather, external field, Boris push (unless FROZEN) and move of one particle.  On return d
-// holds the push displacement (cells), s the cell shift, o1 the new offsets and c the new cell.
-// Returns false when the particle left through a non-periodic face (it becomes a dummy).
-template <int ORDER, bool FROZEN, class Acc, int GATHER = 0>
-__device__ __forceinline__ bool push_move(Acc &acc, const float o[3], int c[3], float4 &mo,
-                                          const SpeciesDev &sp, const GridDev &g, const ExtDev &ext,
-                                          int *err, float d[3], int s[3], float o1[3], int zb)
+// Gather, external field and Boris rotation of one particle: u^{n-1/2} -> u^{n+1/2} in mo.
+// GATHER 0: momentum-conserving (the deposit's shape at each component's Yee point); GATHER 1:
+// energy-conserving (one order lower along the component's staggered dims: the transpose of the
+// Esirkepov deposit, whose J_x has the lower-order shape at the half-integer x nodes).
+template <int ORDER, class Acc, int GATHER = 0>
+__device__ __forceinline__ void push_u(Acc &acc, const float o[3], const int c[3], float4 &mo,
+                                       const SpeciesDev &sp, const ExtDev &ext)
 {
-    if (!FROZEN) push_u<ORDER, Acc, GATHER>(acc, o, c, mo, sp, ext);
+    using S = Shape<ORDER>;
+    using SS = Shape<GATHER ? ORDER - 1 : ORDER>;   // shape along staggered dims
+    constexpr int N = S::N, NS = SS::N;
+    int su[3], ss[3];
+    float wu[3][N], ws[3][NS];
+#pragma unroll
+    for (int dd = 0; dd < 3; dd++) { S::unst(o[dd], su[dd], wu[dd]); SS::stag(o[dd], ss[dd], ws[dd]); }
+    float E[3], B[3];
+    acc.template gather_windows<N, NS>(su, ss);
+    E[0] = gather3<true, false, false, N, NS>(acc, 0, su, ss, wu, ws);
+    E[1] = gather3<false, true, false, N, NS>(acc, 1, su, ss, wu, ws);
+    E[2] = gather3<false, false, true, N, NS>(acc, 2, su, ss, wu, ws);
+    B[0] = gather3<false, true, true, N, NS>(acc, 3, su, ss, wu, ws);
+    B[1] = gather3<true, false, true, N, NS>(acc, 4, su, ss, wu, ws);
+    B[2] = gather3<true, true, false, N, NS>(acc, 5, su, ss, wu, ws);
+    kick(o, c, E, B, mo, sp, ext);
+}
+
+// Move of one particle: d the displacement (cells), s the cell shift, o1 the new offsets and c the
+// new cell.  False when the particle left through a non-periodic face or its momentum is not finite
+// (it becomes a dummy).
+__device__ __forceinline__ bool move(const float o[3], int c[3], const float4 &mo, const GridDev &g, int *err, float d[3],
+                                     int s[3], float o1[3], int zb)
+{
     const float u[3] = {mo.x, mo.y, mo.z};
     const float ig = rsqrtf(1.f + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
     if (!(ig > 0.f)) { atomicOr(err, ERR_NAN); return false; }
     bool alive = true;
 #pragma unroll
     for (int dd = 0; dd < 3; dd++) {
-        d[dd] = u[dd] * ig * g.dt_over_d[dd];        // displacement of the push (cells)
-        const float x1 = o[dd] + d[dd];
+        // the displacement of the push (cells), and the new offset with one rounding; both are spelt
+        // out, so that every path (and build) moves a particle to the same place: a cold lattice's
+        // particles round alike, and a neutral plasma's current is a small difference of large ones
+        const float v = __fmul_rn(u[dd], ig);
+        d[dd] = __fmul_rn(v, g.dt_over_d[dd]);
+        const float x1 = fmaf(v, g.dt_over_d[dd], o[dd]);
         s[dd] = (int)floorf(x1);
         o1[dd] = x1 - (float)s[dd];
         if (o1[dd] >= 1.f) { o1[dd] = 0.f; s[dd] += 1; }
@@ -514,6 +525,24 @@ __device__ __forceinline__ bool push_move(Acc &acc, const float o[3], int c[3], 
     return alive;
 }
 
+// Gather, external field, push (unless FROZEN) and move of one particle (see move).
+template <int ORDER, bool FROZEN, class Acc, int GATHER = 0>
+__device__ __forceinline__ bool push_move(Acc &acc, const float o[3], int c[3], float4 &mo,
+                                          const SpeciesDev &sp, const GridDev &g, const ExtDev &ext,
+                                          int *err, float d[3], int s[3], float o1[3], int zb)
+{
+    if (!FROZEN) push_u<ORDER, Acc, GATHER>(acc, o, c, mo, sp, ext);
+    return move(o, c, mo, g, err, d, s, o1, zb);
+}
+
+// First node of the general deposit window, relative to the cell.
+template <int ORDER> __device__ __forceinline__ int general_start(float o, float d, int s)
+{
+    if (ORDER == 1) return min(s, 0);
+    const int b0 = o >= 0.5f, b1 = (int)floorf(o + d + 0.5f);
+    return b0 - 1 + min(b1 - b0, 0);
+}
+
 template <int ORDER>
 __device__ __forceinline__ bool stays_all(const float o[3], const float d[3], const int s[3])
 {
@@ -521,15 +550,13 @@ __device__ __forceinline__ bool stays_all(const float o[3], const float d[3], co
            Shape<ORDER>::stays(o[2], d[2], s[2]);
 }
 
-// Whole step of one particle on the global-memory path.
+// Whole step of one particle's record on the global-memory path; dmax (may be NULL) takes the
+// largest displacement per component (float bits).
 template <int ORDER, bool FROZEN, int GATHER = 0>
-__device__ __forceinline__ void step_global(const SpeciesDev &sp, const GridDev &g, const FieldsDev &f,
-                                            const ExtDev &ext, int *err, int p)
+__device__ __forceinline__ void step_record(float4 &P, float4 &mo, const SpeciesDev &sp, const GridDev &g, const FieldsDev &f,
+                                            const ExtDev &ext, int *err, unsigned *dmax)
 {
-    float4 P = sp.pos[p];
     const int cell = __float_as_int(P.w);
-    if (cell < 0) return;
-    float4 mo = sp.mom[p];
     int c[3] = {g.cc.i(cell), g.cc.j(cell), g.cc.k(cell)};
     const float o[3] = {P.x, P.y, P.z};
     const int zb = g.nzr == g.n[2] ? 0 : zblock(c[2], g.nzr);
@@ -540,39 +567,29 @@ __device__ __forceinline__ void step_global(const SpeciesDev &sp, const GridDev 
         const float fac[3] = {sp.cf[0] * mo.w, sp.cf[1] * mo.w, sp.cf[2] * mo.w};
         deposit_general<ORDER>(acc, o, d, s, fac);
         P = make_float4(o1[0], o1[1], o1[2], __int_as_float(g.cc.pack(c[0], c[1], c[2])));
-        if (!FROZEN) sp.mom[p] = mo;
+        if (dmax)
+#pragma unroll
+            for (int k = 0; k < 3; k++) dmax[k] = max(dmax[k], __float_as_uint(fabsf(d[k])));
     } else {
         P.w = __int_as_float(-1);
     }
+}
+
+template <int ORDER, bool FROZEN, int GATHER = 0>
+__device__ __forceinline__ void step_global(const SpeciesDev &sp, const GridDev &g, const FieldsDev &f,
+                                            const ExtDev &ext, int *err, int p)
+{
+    float4 P = sp.pos[p];
+    if (__float_as_int(P.w) < 0) return;
+    float4 mo = sp.mom[p];
+    step_record<ORDER, FROZEN, GATHER>(P, mo, sp, g, f, ext, err, nullptr);
+    if (!FROZEN) sp.mom[p] = mo;
     sp.pos[p] = P;
 }
 
 // Linear index of grid node (x, y, z) with periodic wrap (z inside the run starting at row zb),
 // or -1 outside a non-periodic face.
 __device__ __forceinline__ long long wrap_node(const GridDev &g, int x, int y, int z, int zb);
-
-// Stage the six field components of a tile's region in shared memory.  A tile away from every
-// face needs no wrap or bounds test; the loop runs over the region's nodes with compile-time
-// divisions (fixed region) and each thread moves all components of its node.
-template <class Reg>
-__device__ __forceinline__ void stage_fields(const Reg &reg, const GridDev &g, const FieldsDev &f, float *sF,
-                                             const int reg0[3], bool interior, long long gbase, int zb)
-{
-    const int Rx = reg.rx(), Ry = reg.ry(), R2 = reg.r2(), R3 = reg.r3();
-    const long long gnx = g.n[0], gnxy = (long long)g.n[0] * g.n[1];
-    for (int l = threadIdx.x; l < R3; l += blockDim.x) {
-        const int lz = l / R2, rem = l - lz * R2, ly = rem / Rx, lx = rem - ly * Rx;
-        if (ly >= Ry) continue;   // plane padding
-        const long long gi = interior ? gbase + lz * gnxy + ly * gnx + lx
-                                      : wrap_node(g, reg0[0] + lx, reg0[1] + ly, reg0[2] + lz, zb);
-#pragma unroll
-        for (int comp = 0; comp < 3; comp++) {
-            sF[comp * R3 + l] = gi >= 0 ? __ldg(f.E + comp * g.ncell + gi) : 0.f;
-            sF[(comp + 3) * R3 + l] = gi >= 0 ? __ldg(f.B + comp * g.ncell + gi) : 0.f;
-        }
-    }
-}
-
 
 __device__ __forceinline__ long long wrap_node(const GridDev &g, int x, int y, int z, int zb)
 {
@@ -593,9 +610,9 @@ __device__ __forceinline__ long long wrap_node(const GridDev &g, int x, int y, i
 
 // One CTA of kPushThreads per SM: the shared region of a tile holds most of the SM's shared
 // memory, and 1024 threads at 64 registers (a few spills) hide more latency than 512 at 122.
-template <int ORDER, bool FROZEN, class Reg, int GATHER>
+template <int ORDER, class Reg>
 __global__ void __launch_bounds__(kPushThreads, 1)
-k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work, int *work_sparse, int *err, Reg reg)
+k_push_frozen(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work, int *work_sparse, int *err, Reg reg)
 {
     const ExtDev ext = ext_at_clock(ext0);
     extern __shared__ float smem[];
@@ -603,8 +620,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
     __shared__ float s_js[3], s_jinv[3], s_dl[3];
     __shared__ unsigned s_dm[3];
     const int Rx = reg.rx(), R3 = reg.r3();
-    float *sF = smem;
-    unsigned *sJlo = reinterpret_cast<unsigned *>(FROZEN ? smem : smem + 6 * R3);
+    unsigned *sJlo = reinterpret_cast<unsigned *>(smem);
     int *sJhi = reinterpret_cast<int *>(sJlo + 3 * R3);
     int *qb = sJhi + 3 * R3;                              // queue: local base index
     float *qd = reinterpret_cast<float *>(qb + kQueue);  // queue: o[3], d[3], w (SoA)
@@ -624,17 +640,16 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             const int p_begin = n_sorted + (item - n_tile_items) * chunk;
             const int p_end = min(p_begin + chunk, n_total);
             for (int p = p_begin + threadIdx.x; p < p_end; p += blockDim.x)
-                step_global<ORDER, FROZEN, GATHER>(sp, g, f, ext, err, p);
+                step_global<ORDER, true>(sp, g, f, ext, err, p);
             continue;
         }
 
-        const int2 wi = t.items[item];
+        const int4 wi = t.items[item];
         const int tile = wi.x;
         const int tx = tile % t.nt[0], ty = (tile / t.nt[0]) % t.nt[1], tz = tile / (t.nt[0] * t.nt[1]);
         const int t0[3] = {tx * t.T[0], ty * t.T[1], tz * t.T[2]};
         const int reg0[3] = {t0[0] - t.M - t.hl, t0[1] - t.M - t.hl, t0[2] - t.M - t.hl};
-        const int p_begin = t.tile_start[tile] + wi.y * chunk;
-        const int p_end = min(p_begin + chunk, t.tile_start[tile + 1]);
+        const int p_begin = wi.y, p_end = wi.z;
         // Region of the tile: nodes reg0 + (0..R-1) per dim (plane pitch padded).
         const int R2 = reg.r2(), Ry = reg.ry(), Rz = R3 / R2;
         const int zb = g.nzr == g.n[2] ? 0 : zblock(t0[2], g.nzr);   // the tile's run (tiles never straddle runs)
@@ -642,7 +657,6 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
                               reg0[2] >= zb && reg0[2] + Rz <= zb + g.nzr;
         const long long gnx = g.n[0], gnxy = (long long)g.n[0] * g.n[1];
         const long long gbase = reg0[2] * gnxy + reg0[1] * gnx + reg0[0];
-        if (!FROZEN) stage_fields(reg, g, f, sF, reg0, interior, gbase, zb);
         for (int l = threadIdx.x; l < 3 * R3; l += blockDim.x) {
             sJlo[l] = 0u;
             sJhi[l] = 0;
@@ -701,16 +715,16 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
                 fast = fast && r >= -t.M && r < t.T[dd] + t.M;
             }
             if (!fast) {
-                step_global<ORDER, FROZEN, GATHER>(sp, g, f, ext, err, p);
+                step_global<ORDER, true>(sp, g, f, ext, err, p);
                 break;
             }
             float4 mo = sp.mom[p];
             const float o[3] = {P.x, P.y, P.z};
             const int base = (rel[2] + t.M + t.hl) * reg.r2() + (rel[1] + t.M + t.hl) * Rx + rel[0] + t.M + t.hl;
-            SmemAcc<Reg> acc{reg, sF, sJlo, sJhi, s_js, base};
+            SmemAcc<Reg> acc{reg, nullptr, sJlo, sJhi, s_js, base};
             float d[3], o1[3];
             int s[3];
-            if (push_move<ORDER, FROZEN, SmemAcc<Reg>, GATHER>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb)) {
+            if (push_move<ORDER, true, SmemAcc<Reg>>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb)) {
                 const float fac[3] = {sp.cf[0] * mo.w, sp.cf[1] * mo.w, sp.cf[2] * mo.w};
 #pragma unroll
                 for (int k = 0; k < 3; k++) dm[k] = __float_as_uint(fabsf(d[k]));
@@ -738,7 +752,6 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
                     }
                 }
                 P = make_float4(o1[0], o1[1], o1[2], __int_as_float(g.cc.pack(c[0], c[1], c[2])));
-                if (!FROZEN) sp.mom[p] = mo;
             } else {
                 P.w = __int_as_float(-1);
             }
@@ -769,7 +782,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
                 if (x1 - (float)s[dd] >= 1.f) s[dd] += 1;
             }
             const float fac[3] = {sp.cf[0] * w, sp.cf[1] * w, sp.cf[2] * w};
-            SmemAcc<Reg> acc{reg, sF, sJlo, sJhi, s_js, qb[q]};
+            SmemAcc<Reg> acc{reg, nullptr, sJlo, sJhi, s_js, qb[q]};
             deposit_general<ORDER>(acc, o, d, s, fac);
         }
         __syncthreads();
@@ -803,7 +816,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
         if (it >= n_sparse) break;
         const int tile = t.sparse_tiles[it];
         const int pe = t.tile_start[tile + 1];
-        for (int p = t.tile_start[tile] + lane; p < pe; p += 32) step_global<ORDER, FROZEN, GATHER>(sp, g, f, ext, err, p);
+        for (int p = t.tile_start[tile] + lane; p < pe; p += 32) step_global<ORDER, true>(sp, g, f, ext, err, p);
     }
 }
 
@@ -819,53 +832,44 @@ static __global__ void k_dlim_update(float *dlim, unsigned *dmax, float l0, floa
     dmax[k] = 0u;
 }
 
-template <int ORDER, bool FROZEN, int GATHER, class Reg>
-cudaError_t launch_t(pic_ctx *c, int si, const ExtDev &ext, Reg reg, int R3)
-{
-    const Species &s = c->sp[si];
-    TileDev t = tile_dev(c, s);
-    const size_t smem = (size_t)(FROZEN ? 0 : 6) * R3 * sizeof(float) + (size_t)3 * R3 * 2 * sizeof(int) +
-                        (size_t)kQueue * 8 * sizeof(float);
-    auto kern = k_push<ORDER, FROZEN, Reg, GATHER>;
-    // attribute and occupancy once per kernel and region size (nothing but launches is then issued
-    // while a step sequence is captured into a CUDA graph).  The cache is shared by every context
-    // of the process: host threads driving contexts at once take it under a lock, and the shared-
-    // memory attribute only grows, so a launch issued after the lock is released never meets a
-    // smaller limit set by another thread.
-    constexpr int kMaxDevices = 64;
-    static std::mutex mu;
-    static size_t attr_max[kMaxDevices] = {};
-    static size_t occ_smem = 0;
-    static int occ_dev = -1, occ_per_sm = 0;
-    cudaError_t e = cudaSuccess;
-    int per_sm = 0;
+// Launch of a particle kernel: the shared-memory attribute and the occupancy are looked up once per
+// kernel and size (nothing but launches is then issued while a step sequence is captured into a CUDA
+// graph).  The cache is shared by every context of the process: host threads driving contexts at
+// once take it under a lock, and the shared-memory attribute only grows, so a launch issued after
+// the lock is released never meets a smaller limit set by another thread.
+struct KernelCache {
+    static constexpr int kMaxDevices = 64;
+    std::mutex mu;
+    size_t attr_max[kMaxDevices] = {};
+    size_t occ_smem = 0;
+    int occ_dev = -1, occ_per_sm = 0;
+    cudaError_t blocks_per_sm(const void *kern, int dv, int threads, size_t smem, int *per_sm)
     {
         std::lock_guard<std::mutex> lk(mu);
-        const int dv = c->dev.device;
         if (dv < 0 || dv >= kMaxDevices) return cudaErrorInvalidDevice;
+        cudaError_t e;
         if (attr_max[dv] < smem) {
             e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
             attr_max[dv] = smem;
         }
         if (occ_smem != smem || occ_dev != dv) {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_per_sm, kern, kPushThreads, smem);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_per_sm, kern, threads, smem);
             if (e != cudaSuccess) return e;
             occ_smem = smem;
             occ_dev = dv;
         }
-        per_sm = occ_per_sm;
+        *per_sm = occ_per_sm;
+        return occ_per_sm < 1 ? cudaErrorInvalidConfiguration : cudaSuccess;
     }
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    FieldsDev f{c->E, c->B, c->J};
-    kern<<<c->num_sms * per_sm, kPushThreads, smem, c->stream>>>(species_dev(c, s), grid_dev(c), t, f, ext,
-                                                                   c->work + si, c->work + kMaxSpecies + si, c->err,
-                                                                   reg);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+};
+
+inline cudaError_t launch_dlim_update(pic_ctx *c, const Species &s)
+{
     float light[3];
     for (int d = 0; d < 3; d++) light[d] = (float)std::min(1.0, c->dt / c->d[d]);
     k_dlim_update<<<1, 32, 0, c->stream>>>(s.dlim, s.dmax, light[0], light[1], light[2]);
-    c->kernels += 2;
+    c->kernels += 2;   // with the particle kernel before it
     return cudaGetLastError();
 }
 
@@ -876,36 +880,33 @@ inline bool default_region(const pic_ctx *c)
     return c->T[0] == 8 && c->T[1] == 8 && c->T[2] == 8 && c->M == 1;
 }
 
-// One kernel variant: shape order, frozen or mobile species, compile-time (FIXED) or runtime
-// region, gather scheme (mobile species).  The second-order variants each sit in a translation
-// unit of their own, so that the build compiles them in parallel.
-template <int ORDER, bool FROZEN, bool FIXED, int GATHER = 0>
-cudaError_t launch_variant(pic_ctx *c, int si, const ExtDev &ext)
+template <int ORDER, class Reg>
+cudaError_t launch_frozen_t(pic_ctx *c, int si, const ExtDev &ext, Reg reg, int R3)
 {
-    if constexpr (FIXED) {
-        constexpr int R = 8 + 2 * 1 + (ORDER == 1 ? 3 : 5);
-        RegFix<R, R, R> reg;
-        constexpr int R3 = plane_pitch(R, R) * R;
-        return launch_t<ORDER, FROZEN, GATHER>(c, si, ext, reg, R3);
-    } else {
-        const TileDev t = tile_dev(c, c->sp[si]);
-        const int P2 = plane_pitch(t.R[0], t.R[1]);
-        RegDyn reg{t.R[0], t.R[1], P2, P2 * t.R[2]};
-        return launch_t<ORDER, FROZEN, GATHER>(c, si, ext, reg, reg.R3);
-    }
+    static KernelCache cache;
+    const Species &s = c->sp[si];
+    const size_t smem = (size_t)3 * R3 * 2 * sizeof(int) + (size_t)kQueue * 8 * sizeof(float);
+    auto kern = k_push_frozen<ORDER, Reg>;
+    int per_sm = 0;
+    cudaError_t e = cache.blocks_per_sm((const void *)kern, c->dev.device, kPushThreads, smem, &per_sm);
+    if (e != cudaSuccess) return e;
+    kern<<<c->num_sms * per_sm, kPushThreads, smem, c->stream>>>(species_dev(c, s), grid_dev(c), tile_dev(c, s),
+                                                                  FieldsDev{c->E, c->B, c->J}, ext, c->work + si,
+                                                                  c->work + kMaxSpecies + si, c->err, reg);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_dlim_update(c, s);
 }
 
-template <int ORDER>
-cudaError_t launch_order(pic_ctx *c, int si, const ExtDev &ext)
+// Frozen species: the region spans the tile, its drift margin and the general deposit window.
+template <int ORDER> cudaError_t launch_frozen(pic_ctx *c, int si, const ExtDev &ext)
 {
-    const bool fr = c->sp[si].frozen != 0;
-    const bool ec = c->gather == PIC_GATHER_ENERGY;
     if (default_region(c)) {
-        if (fr) return launch_variant<ORDER, true, true>(c, si, ext);
-        return ec ? launch_variant<ORDER, false, true, 1>(c, si, ext) : launch_variant<ORDER, false, true>(c, si, ext);
+        constexpr int R = 8 + 2 * 1 + (ORDER == 1 ? 3 : 5);
+        return launch_frozen_t<ORDER>(c, si, ext, RegFix<R, R, R>{}, plane_pitch(R, R) * R);
     }
-    if (fr) return launch_variant<ORDER, true, false>(c, si, ext);
-    return ec ? launch_variant<ORDER, false, false, 1>(c, si, ext) : launch_variant<ORDER, false, false>(c, si, ext);
+    const TileDev t = tile_dev(c, c->sp[si]);
+    const int P2 = plane_pitch(t.R[0], t.R[1]);
+    return launch_frozen_t<ORDER>(c, si, ext, RegDyn{t.R[0], t.R[1], P2, P2 * t.R[2]}, P2 * t.R[2]);
 }
 
 }  // namespace push

@@ -1,0 +1,435 @@
+// Particle kernel of the mobile species (sm_103a): gather, external field, push, move and Esirkepov
+// deposit.
+#pragma once
+
+#include "push_impl.cuh"
+
+namespace gbpic {
+namespace push {
+
+__device__ __forceinline__ void cp_async4(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Deposit of a particle whose nearest node (TSC) or cell (CIC) changes along one dim only (e): the
+// window is a node longer along e than the simple one and as long along the two others, 75 nodes for
+// TSC against the general window's 144 and without the general window's tests at every node.  The
+// dims are taken in the cyclic order e, e + 1, e + 2 with their strides, so one code serves all.
+template <int ORDER, class Reg>
+__device__ __forceinline__ void deposit_cross(const SmemAcc<Reg> &acc, const float o[3], const float d[3], const int s[3],
+                                              const float fac[3], int e)
+{
+    using S = Shape<ORDER>;
+    constexpr int L = S::L, N = S::N;
+    const int stride[3] = {1, acc.reg.rx(), acc.reg.r2()};
+    const int a = e == 2 ? 0 : e + 1, b = a == 2 ? 0 : a + 1;
+    auto pickf = [](const auto *v, int i) { return i == 0 ? v[0] : (i == 1 ? v[1] : v[2]); };
+    const int se = pickf(stride, e), sa = pickf(stride, a), sb = pickf(stride, b);
+    const float oe = pickf(o, e), de = pickf(d, e);
+    const int she = pickf(s, e);
+    float S0e[L], De[L], S0a[N], Da[N], S0b[N], Db[N];
+    int ste, sta, stb;
+    S::general(oe, de, she, ste, S0e, De);
+    S::simple(pickf(o, a), pickf(d, a), sta, S0a, Da);
+    S::simple(pickf(o, b), pickf(d, b), stb, S0b, Db);
+    float Ae[L], Qe[L], Fe[L - 1], Aa[N], Qa[N], Fa[N - 1], Ab[N], Qb[N], Fb[N - 1];
+    const float fe = pickf(fac, e) * acc.scale(e), fa = pickf(fac, a) * acc.scale(a), fb = pickf(fac, b) * acc.scale(b);
+    float run = 0.f;
+#pragma unroll
+    for (int i = 0; i < L; i++) {
+        Ae[i] = fmaf(0.5f, De[i], S0e[i]);
+        Qe[i] = De[i] * (1.f / 12.f);
+        run += De[i];
+        if (i < L - 1) Fe[i] = fe * run;
+    }
+    float ra = 0.f, rb = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; i++) {
+        Aa[i] = fmaf(0.5f, Da[i], S0a[i]);
+        Qa[i] = Da[i] * (1.f / 12.f);
+        Ab[i] = fmaf(0.5f, Db[i], S0b[i]);
+        Qb[i] = Db[i] * (1.f / 12.f);
+        ra += Da[i];
+        rb += Db[i];
+        if (i < N - 1) { Fa[i] = fa * ra; Fb[i] = fb * rb; }
+    }
+    const int at = acc.base + ste * se + sta * sa + stb * sb;
+    const int pe = at + e * acc.reg.r3(), pa = at + a * acc.reg.r3(), pb = at + b * acc.reg.r3();
+#pragma unroll
+    for (int m = 0; m < N; m++)
+#pragma unroll
+        for (int l = 0; l < N; l++) {
+            const float Y = fmaf(Aa[l], Ab[m], Qa[l] * Db[m]);
+#pragma unroll
+            for (int k = 0; k < L - 1; k++) acc.add(pe + k * se + l * sa + m * sb, Fe[k] * Y);
+        }
+#pragma unroll
+    for (int m = 0; m < L; m++)
+#pragma unroll
+        for (int l = 0; l < N; l++) {
+            const float Ya = fmaf(Ab[l], Ae[m], Qb[l] * De[m]);       // J_a: a; b, e
+            const float Yb = fmaf(Ae[m], Aa[l], Qe[m] * Da[l]);       // J_b: b; e, a
+#pragma unroll
+            for (int k = 0; k < N - 1; k++) {
+                acc.add(pa + k * sa + l * sb + m * se, Fa[k] * Ya);
+                acc.add(pb + k * sb + l * sa + m * se, Fb[k] * Yb);
+            }
+        }
+}
+
+constexpr int kList = kChunk;   // a record is listed once at most
+constexpr int kMobileThreads = 512;
+
+// ------------------------------------------------------------------ the kernel
+// A work item is up to kChunk particles of one tile.  Its E and B region is staged in shared memory
+// and its current summed there in fixed point (see SmemAcc), as for the frozen species; a thread
+// takes one particle at a time.  The bound is the shared-memory and L1 pipe together with issue: per
+// particle 162 field loads, 108 atomics and the records' lines against ~1,500 thread instructions.
+//  - Lanes: the sort leaves a tile's particles octant by octant along its rows (tile_key), so that
+//    32 consecutive records of a lattice are on 32 cells at the same place in their cells.  Lane l
+//    takes record l K + k, K the records of an octant in an even tile: for K = 1 a warp's records
+//    fill whole lines and its 8 x 4 cells 32 different banks (push_pitch); a denser tile spreads its
+//    lanes over more cells instead of queueing them on the same words.  With the records of a cell
+//    together (lanes 128 records apart) every record was a line of its own, one line a clock, and
+//    field loads and atomics met 1.5 and 1.7 times: 20 clocks a particle on that pipe, now 13.
+//  - The region spans the nodes that gathers and simple deposits touch, a node less on each side
+//    than the general deposit window needs (13^3 instead of 15^3 for TSC on 8^3 cells).
+//  - The region starts at the tile's edge less the margin unless the particles can have drifted
+//    further than that since the sort: it then follows the item's particles, as long as they fit.
+//  - Particles whose nearest node changes in the step are listed and taken after the others, a thread
+//    each: nearly all change it along one dim (deposit_cross).  So are particles outside the region,
+//    through global memory.
+// 512 threads at 128 registers against 1024 at 64, in ms per step: plasma buncher 4.15 and 4.08, 64
+// runs of the sweep 15.1 and 14.9, 300k electrons on 45 x 39 x 70 cells 0.114 and 0.126, 65k CIC 0.046
+// and 0.051.
+template <int ORDER, int GATHER, int NT, int MINB, class Reg>
+__global__ void __launch_bounds__(NT, MINB)
+k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work, int *work_sparse, int *err, Reg reg, int age)
+{
+    using S = Shape<ORDER>;
+        const ExtDev ext = ext_at_clock(ext0);
+    extern __shared__ __align__(16) float smem[];
+    __shared__ int4 s_item;
+    __shared__ float s_js[3], s_jinv[3], s_dl[3];
+    __shared__ int s_lo[3], s_hi[3], s_sum[3], s_live, s_n1, s_n2;
+    const int Rx = reg.rx(), Ry = reg.ry(), R2 = reg.r2(), R3 = reg.r3(), Rz = R3 / R2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // shared memory: the currents' words, the fields, the list (records outside the region from the
+    // front, pushed records whose deposit is due from the back)
+    unsigned *sJlo = reinterpret_cast<unsigned *>(smem);
+    int *sJhi = reinterpret_cast<int *>(sJlo + 3 * R3);
+    float *sF = reinterpret_cast<float *>(sJhi + 3 * R3);
+    unsigned short *list = reinterpret_cast<unsigned short *>(sF + 6 * R3);
+
+    const int n_total = sp.count[0], n_sorted = sp.count[1], n_items = sp.count[2];
+    const long long gnx = g.n[0], gnxy = (long long)g.n[0] * g.n[1];
+    unsigned dmax[3] = {0u, 0u, 0u};
+
+    for (;;) {
+        __syncthreads();                           // the last item's flush has read its currents
+        if (tid == 0) {
+            const int it = atomicAdd(work, 1);
+            s_item = it < n_items ? t.items[it] : make_int4(-1, 0, 0, 0);
+            s_n1 = 0;
+            s_n2 = 0;
+            s_live = 0;
+        }
+        if (tid < 3) {
+            s_lo[tid] = 1 << 20;
+            s_hi[tid] = -(1 << 20);
+            s_sum[tid] = 0;
+        }
+        for (int l = tid; l < 6 * R3; l += NT) sJlo[l] = 0u;   // both words
+        __syncthreads();
+        const int4 item = s_item;
+        if (item.x < 0) break;
+        const int tile = item.x, p0 = item.y, p1 = item.z;
+        const int t0[3] = {(tile % t.nt[0]) * t.T[0], ((tile / t.nt[0]) % t.nt[1]) * t.T[1], (tile / (t.nt[0] * t.nt[1])) * t.T[2]};
+        const int zb = g.nzr == g.n[2] ? 0 : zblock(t0[2], g.nzr);
+        // cell coordinates relative to the tile (the nearest periodic image)
+        auto relative = [&](int cell, int rel[3]) {
+            const int c[3] = {g.cc.i(cell), g.cc.j(cell), g.cc.k(cell)};
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                int r = c[d] - t0[d];
+                if (g.periodic[d]) {
+                    const int per = d == 2 ? g.nzr : g.n[d];
+                    if (r > per / 2) r -= per;
+                    else if (r < -per / 2) r += per;
+                }
+                rel[d] = r;
+            }
+        };
+        if (tid < 3) {
+            // fixed-point scale of the item: the largest contribution jb w dlim maps to <= 2^30
+            const float w = sp.wrun ? sp.wrun[t0[2] / g.nzr] : sp.wmax;
+            const float dl = sp.dlim[tid];
+            const float bd = sp.jb[tid] * w * dl;
+            int e = 0;
+            frexpf(bd, &e);                       // bd < 2^e
+            const int ex = bd > 0.f ? min(max(30 - e, -100), 100) : 0;
+            s_js[tid] = ldexpf(1.f, ex);
+            s_jinv[tid] = ldexpf(1.f, -ex);
+            s_dl[tid] = dl;
+        }
+        int org[3] = {-t.M, -t.M, -t.M};
+        // dlim is four times the last step's largest displacement
+        const float reach = 0.25f * (float)age * fmaxf(sp.dlim[0], fmaxf(sp.dlim[1], sp.dlim[2]));
+        if (reach > (float)t.M) {
+            int lo[3] = {1 << 20, 1 << 20, 1 << 20}, hi[3] = {-(1 << 20), -(1 << 20), -(1 << 20)}, sum[3] = {0, 0, 0}, live = 0;
+            for (int p = p0 + tid; p < p1; p += NT) {
+                const int cell = __float_as_int(sp.pos[p].w);
+                if (cell < 0) continue;
+                int rel[3];
+                relative(cell, rel);
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    lo[d] = min(lo[d], rel[d]);
+                    hi[d] = max(hi[d], rel[d]);
+                    sum[d] += rel[d];
+                }
+                live++;
+            }
+            live = __reduce_add_sync(0xffffffffu, live);
+            if (lane == 0) atomicAdd(&s_live, live);
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                lo[d] = __reduce_min_sync(0xffffffffu, lo[d]);
+                hi[d] = __reduce_max_sync(0xffffffffu, hi[d]);
+                sum[d] = __reduce_add_sync(0xffffffffu, sum[d]);
+                if (lane == 0) {
+                    atomicMin(&s_lo[d], lo[d]);
+                    atomicMax(&s_hi[d], hi[d]);
+                    atomicAdd(&s_sum[d], sum[d]);
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                const int w = t.T[d] + 2 * t.M, l = s_lo[d], h = s_hi[d];
+                if (h < l) continue;
+                if (h - l + 1 > w) org[d] = (int)floorf((float)s_sum[d] / (float)s_live + 1.f) - w / 2;   // about their mean
+                else if (l < org[d]) org[d] = l;
+                else if (h >= org[d] + w) org[d] = h - w + 1;
+            }
+        }
+        const int reg0[3] = {t0[0] + org[0] - 1, t0[1] + org[1] - 1, t0[2] + org[2] - 1};
+        const bool interior = reg0[0] >= 0 && reg0[0] + Rx <= g.n[0] && reg0[1] >= 0 && reg0[1] + Ry <= g.n[1] &&
+                              reg0[2] >= zb && reg0[2] + Rz <= zb + g.nzr;
+        const long long gbase = reg0[2] * gnxy + reg0[1] * gnx + reg0[0];
+        auto node = [&](int l) {
+            const int lz = l / R2, rem = l - lz * R2, ly = rem / Rx, lx = rem - ly * Rx;
+            if (ly >= Ry) return -1ll;               // plane padding
+            return interior ? gbase + lz * gnxy + ly * gnx + lx : wrap_node(g, reg0[0] + lx, reg0[1] + ly, reg0[2] + lz, zb);
+        };
+        for (int l = tid; l < R3; l += NT) {
+            const long long gi = node(l);
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                if (gi >= 0) {
+                    cp_async4(sF + c * R3 + l, f.E + c * g.ncell + gi);
+                    cp_async4(sF + (c + 3) * R3 + l, f.B + c * g.ncell + gi);
+                } else {
+                    sF[c * R3 + l] = 0.f;
+                    sF[(c + 3) * R3 + l] = 0.f;
+                }
+            }
+        }
+        cp_async_wait();
+        __syncthreads();
+
+        // region coordinates of a cell: true inside the region
+        auto in_region = [&](int cell, int rel[3]) {
+            relative(cell, rel);
+            bool in = true;
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                rel[d] -= org[d];
+                in = in && (unsigned)rel[d] < (unsigned)(t.T[d] + 2 * t.M);
+                rel[d] += 1;
+            }
+            return in;
+        };
+        const int tile_n = t.tile_start[tile + 1] - t.tile_start[tile], len = p1 - p0;
+        const int K = max(1, min((tile_n + 4 * t.tile_cells) / (8 * t.tile_cells), (len + 31) / 32));
+        const int rounds = (len + 32 * K - 1) / (32 * K) * K;
+        for (int rd = warp; rd < rounds; rd += NT / 32) {
+            const int q = (rd / K) * 32 * K + lane * K + rd % K;
+            if (q >= len) continue;
+            const int p = p0 + q;
+            const float4 R = sp.pos[p];
+            const int cell = __float_as_int(R.w);
+            if (cell < 0) continue;
+            int rel[3];
+            if (!in_region(cell, rel)) {
+                list[atomicAdd(&s_n1, 1)] = (unsigned short)q;
+                continue;
+            }
+            float4 mo = sp.mom[p];
+            const float o[3] = {R.x, R.y, R.z};
+            int c[3] = {g.cc.i(cell), g.cc.j(cell), g.cc.k(cell)}, s[3];
+            SmemAcc<Reg> acc{reg, sF, sJlo, sJhi, s_js, rel[2] * R2 + rel[1] * Rx + rel[0]};
+            float d[3], o1[3];
+            if (!push_move<ORDER, false, SmemAcc<Reg>, GATHER>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb)) {
+                sp.pos[p].w = __int_as_float(-1);
+                continue;
+            }
+            sp.mom[p] = mo;
+            const bool fits = fabsf(d[0]) <= s_dl[0] && fabsf(d[1]) <= s_dl[1] && fabsf(d[2]) <= s_dl[2];
+            if (!fits || !stays_all<ORDER>(o, d, s)) {
+                list[kList - 1 - atomicAdd(&s_n2, 1)] = (unsigned short)q;   // its position is still the old one
+                continue;
+            }
+            sp.pos[p] = make_float4(o1[0], o1[1], o1[2], __int_as_float(g.cc.pack(c[0], c[1], c[2])));
+#pragma unroll
+            for (int k = 0; k < 3; k++) dmax[k] = max(dmax[k], __float_as_uint(fabsf(d[k])));
+            const float fac[3] = {sp.cf[0] * mo.w, sp.cf[1] * mo.w, sp.cf[2] * mo.w};
+            deposit_simple<ORDER>(acc, o, d, fac);
+        }
+        __syncthreads();
+        // ---- listed records
+        const int n1 = s_n1, n2 = s_n2;
+        for (int q = tid; q < n1 + n2; q += NT) {
+            const int p = p0 + (q < n1 ? list[q] : list[kList - 1 - (q - n1)]);
+            float4 R = sp.pos[p], mo = sp.mom[p];
+            if (q < n1) {
+                step_record<ORDER, false, GATHER>(R, mo, sp, g, f, ext, err, dmax);
+                sp.mom[p] = mo;
+                sp.pos[p] = R;
+                continue;
+            }
+            const int cl = __float_as_int(R.w);
+            int c[3] = {g.cc.i(cl), g.cc.j(cl), g.cc.k(cl)}, s[3], rel[3];
+            const int c0[3] = {c[0], c[1], c[2]};
+            in_region(cl, rel);
+            const float o[3] = {R.x, R.y, R.z};
+            float d[3], o1[3];
+            move(o, c, mo, g, err, d, s, o1, zb);   // it stays in the grid: the first loop's move has seen to that
+            sp.pos[p] = make_float4(o1[0], o1[1], o1[2], __int_as_float(g.cc.pack(c[0], c[1], c[2])));
+            const float fac[3] = {sp.cf[0] * mo.w, sp.cf[1] * mo.w, sp.cf[2] * mo.w};
+            const bool fits = fabsf(d[0]) <= s_dl[0] && fabsf(d[1]) <= s_dl[1] && fabsf(d[2]) <= s_dl[2];
+            bool in = fits;
+            int e = 0, crossed = 0;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                dmax[k] = max(dmax[k], __float_as_uint(fabsf(d[k])));
+                if (S::stays(o[k], d[k], s[k])) continue;
+                e = k;
+                crossed++;
+                const int st = rel[k] + general_start<ORDER>(o[k], d[k], s[k]);
+                in = in && st >= 0 && st + S::L <= (k == 0 ? Rx : (k == 1 ? Ry : Rz));
+            }
+            if (in && crossed == 1) {
+                const SmemAcc<Reg> acc{reg, sF, sJlo, sJhi, s_js, rel[2] * R2 + rel[1] * Rx + rel[0]};
+                deposit_cross<ORDER>(acc, o, d, s, fac, e);
+                continue;
+            }
+            // several dims (its window's tests need every dim), beyond the range or the region
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const int st = rel[k] + general_start<ORDER>(o[k], d[k], s[k]);
+                in = in && st >= 0 && st + S::L <= (k == 0 ? Rx : (k == 1 ? Ry : Rz));
+            }
+            if (in) {
+                SmemAcc<Reg> acc{reg, sF, sJlo, sJhi, s_js, rel[2] * R2 + rel[1] * Rx + rel[0]};
+                deposit_general<ORDER>(acc, o, d, s, fac);
+            } else {
+                GlobAcc<ORDER> acc(f, g, c0, err, zb);
+                deposit_general<ORDER>(acc, o, d, s, fac);
+                if (!fits) atomicAdd(sp.nfall, 1ull);
+            }
+        }
+        __syncthreads();
+        // one flush of the item's current to global memory: hi 2^19 + lo back to float
+        const float jinv[3] = {s_jinv[0], s_jinv[1], s_jinv[2]};
+        for (int l = tid; l < R3; l += NT) {
+            unsigned lo[3];
+            int hi[3];
+            bool have = false;
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                lo[c] = sJlo[c * R3 + l];
+                hi[c] = sJhi[c * R3 + l];
+                have = have || lo[c] != 0u || hi[c] != 0;
+            }
+            if (!have) continue;
+            const long long gi = node(l);
+            if (gi < 0) { atomicOr(err, ERR_INDEX); continue; }   // (plane padding is never written)
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                if (lo[c] == 0u && hi[c] == 0) continue;
+                const float v = fmaf((float)hi[c], (float)(1u << kLoBits), __uint2float_rn(lo[c])) * jinv[c];
+                atomicAdd(f.J + c * g.ncell + gi, v);
+            }
+        }
+    }
+    // the step's largest displacement per component (sets the next step's bound)
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const unsigned m = __reduce_max_sync(0xffffffffu, dmax[k]);
+        if (lane == 0 && m) atomicMax(sp.dmax + k, m);
+    }
+    // appended particles not yet sorted, then sparse tiles (fewer than kSparse particles, a warp
+    // each): staging and flushing a region would cost more than the global path of these few
+    for (int p = n_sorted + blockIdx.x * NT + tid; p < n_total; p += gridDim.x * NT)
+        step_global<ORDER, false, GATHER>(sp, g, f, ext, err, p);
+    const int n_sparse = sp.count[3];
+    for (;;) {
+        int it = 0;
+        if (lane == 0) it = atomicAdd(work_sparse, 1);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= n_sparse) break;
+        const int tile = t.sparse_tiles[it];
+        const int pe = t.tile_start[tile + 1];
+        for (int p = t.tile_start[tile] + lane; p < pe; p += 32) step_global<ORDER, false, GATHER>(sp, g, f, ext, err, p);
+    }
+}
+
+// Plane pitch of the region: rows of a plane's x, the planes 8 (mod 16) words apart, so that the 8 x 4
+// cells of a warp in a full tile sit on 32 banks.
+__host__ __device__ constexpr int push_pitch(int rx, int ry) { return rx * ry + (24 - (rx * ry) % 16) % 16; }
+
+inline size_t push_smem(int R3) { return (size_t)48 * R3 + 2 * kList; }
+
+// Steps since the species' last sort.
+inline int sort_age(const pic_ctx *c) { return (int)((c->step - c->sort_base) % c->sort_every); }
+
+template <int ORDER, int GATHER, int NT, int MINB, class Reg>
+cudaError_t launch_push_t(pic_ctx *c, int si, const ExtDev &ext, Reg reg, int R3)
+{
+    static KernelCache cache;
+    const Species &s = c->sp[si];
+    const size_t smem = push_smem(R3);
+    auto kern = k_push<ORDER, GATHER, NT, MINB, Reg>;
+    int per_sm = 0;
+    cudaError_t e = cache.blocks_per_sm((const void *)kern, c->dev.device, NT, smem, &per_sm);
+    if (e != cudaSuccess) return e;
+    kern<<<c->num_sms * per_sm, NT, smem, c->stream>>>(species_dev(c, s), grid_dev(c), tile_dev(c, s), FieldsDev{c->E, c->B, c->J},
+                                                        ext, c->work + si, c->work + kMaxSpecies + si, c->err, reg, sort_age(c));
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_dlim_update(c, s);
+}
+
+// The region of a tile: its cells and drift margin, one node below and (TSC) two or (CIC) one above.
+template <int ORDER, int GATHER> cudaError_t launch_push_fixed(pic_ctx *c, int si, const ExtDev &ext)
+{
+    constexpr int R = 8 + 2 * 1 + (ORDER == 1 ? 2 : 3), R2 = push_pitch(R, R);
+    return launch_push_t<ORDER, GATHER, kMobileThreads, 1>(c, si, ext, RegFix<R, R, R, R2>{}, R2 * R);
+}
+
+template <int ORDER, int GATHER> cudaError_t launch_push_dyn(pic_ctx *c, int si, const ExtDev &ext)
+{
+    int R[3];
+    for (int d = 0; d < 3; d++) R[d] = c->T[d] + 2 * c->M + (ORDER == 1 ? 2 : 3);
+    const int R2 = push_pitch(R[0], R[1]), R3 = R2 * R[2];
+    const RegDyn reg{R[0], R[1], R2, R3};
+    const size_t smem = push_smem(R3), sm = 228 * 1024, cta = 1024 + 512;
+    if (4 * (smem + cta) <= sm) return launch_push_t<ORDER, GATHER, 128, 4>(c, si, ext, reg, R3);
+    if (2 * (smem + cta) <= sm) return launch_push_t<ORDER, GATHER, 256, 2>(c, si, ext, reg, R3);
+    return launch_push_t<ORDER, GATHER, kMobileThreads, 1>(c, si, ext, reg, R3);
+}
+
+}  // namespace push
+}  // namespace gbpic

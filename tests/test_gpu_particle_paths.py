@@ -62,3 +62,49 @@ def test_particles_drifted_from_their_tiles(order, steps):
     sim, ids = api.from_workload(w, tuning={"tile": (8, 8, 8), "sort_every": 32, "margin": 1})
     sim.step(steps)
     _one_step(w, sim, ids, 7)
+
+
+@pytest.mark.parametrize("order", [1, 2])
+@pytest.mark.parametrize("gather", [0, 1])
+@pytest.mark.parametrize("n", [33, 700, 9000])
+def test_hot_particles_cross_nodes(order, gather, n):
+    # random relativistic momenta: moves of up to 0.28 cells along each dim, so that the nearest node
+    # changes along none, one, two or all dims, in both directions
+    w = W.vacuum_undulator(grid=(20, 10, 18), n_beam=n, seed=3, order=order)
+    w.undulator = None
+    X, U, Wt = W.sample_uniform_particles(w.grid, n, seed=21 + n, umax=4.0)
+    if n == 33:
+        X = 8.0 + 1.5 * (X / np.array(w.grid))      # one tile just above the sparse limit
+    sim, ids = api.from_workload(w, beam=False)
+    ids["beam"] = sim.load_species(-1.0, 1.0, X.T * np.array(w.d)[:, None], U.T, Wt * 1e-3,
+                                   frame=api.PIC_FRAME_BOOSTED)
+    sim.set_gather(gather)
+    _one_step(w, sim, ids, 9, gather)
+
+
+@pytest.mark.parametrize("tile", [(8, 8, 8), (1, 16, 5), (16, 3, 4), (5, 5, 5), (10, 8, 8)])
+@pytest.mark.parametrize("margin", [0, 1, 2])
+def test_tile_shapes_and_margins(tile, margin):
+    # regions of other shapes (one to four CTAs per SM) and drift margins, after five steps of drift
+    w = W.mini_dense_bunch(order=2, n_beam=20000)
+    try:
+        sim, ids = api.from_workload(w, tuning={"tile": tile, "sort_every": 8, "margin": margin})
+    except api.PicError:
+        pytest.skip("the region of this tile exceeds shared memory")
+    sim.step(5)
+    _one_step(w, sim, ids, 13)
+
+
+@pytest.mark.parametrize("order", [1, 2])
+@pytest.mark.parametrize("tile", [(8, 8, 8), (5, 4, 6)])
+def test_frozen_particle_species(order, tile):
+    # a frozen species held as particles (its own kernel) beside a mobile one
+    w = W.vacuum_undulator(grid=(20, 10, 18), n_beam=3000, seed=3, order=order)
+    w.undulator = None
+    sim, ids = api.from_workload(w, beam=False, tuning={"tile": tile, "sort_every": 4, "margin": 1})
+    for name, q, m, seed, frozen in (("plasma_i", 1.0, 1836.15267343, 31, True), ("beam", -1.0, 1.0, 32, False)):
+        X, U, Wt = W.sample_uniform_particles(w.grid, 9000, seed=seed, umax=3.0)
+        ids[name] = sim.load_species(q, m, X.T * np.array(w.d)[:, None], U.T, Wt * 1e-3,
+                                     frame=api.PIC_FRAME_BOOSTED, frozen=frozen)
+    sim.step(2)
+    _one_step(w, sim, ids, 11)
