@@ -136,7 +136,7 @@ struct TileDev {
     const int *cell_start;   // [n_keys + 1]: first sorted slot of each key (8 keys per cell), valid
                              // for the tiles holding particles at the last sort
     const int *tile_start;   // [ntiles + 1]: first sorted slot of each tile (the last: the live count)
-    const int4 *items;       // work items of the tiles with >= kSparse particles: tile, first slot, end slot
+    const int4 *items;       // work items of the tiles with >= kSparse particles: tile, first slot, end slot, particles of the tile
     const int *sparse_tiles; // tiles with 1 .. kSparse-1 particles (count[3] of them)
     int chunk;               // particles per work item (kChunkMin .. kChunk), fixed at the sort
     CellCode cc;

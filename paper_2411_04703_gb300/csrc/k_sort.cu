@@ -179,7 +179,7 @@ __global__ void k_fill_items(const int *chunk_start, const int *sparse_start, in
     if (tl < ntiles) {
         const int b = chunk_start[tl], e = chunk_start[tl + 1];
         const int p0 = tile_start[tl], p1 = tile_start[tl + 1];
-        for (int c = b; c < e; c++) items[c] = make_int4(tl, p0 + (c - b) * chunk, min(p0 + (c - b + 1) * chunk, p1), 0);
+        for (int c = b; c < e; c++) items[c] = make_int4(tl, p0 + (c - b) * chunk, min(p0 + (c - b + 1) * chunk, p1), p1 - p0);
         if (sparse_start[tl + 1] > sparse_start[tl]) sparse_tiles[sparse_start[tl]] = tl;
     }
     if (tl == 0) {
@@ -272,10 +272,13 @@ cudaError_t exclusive_scan(pic_ctx *c, int *data, int64_t n)
 cudaError_t launch_sort(pic_ctx *c, int si, bool by_octant)
 {
     Species &s = c->sp[si];
-    // work items small enough that a small species still gives every SM one (each item stages a
-    // whole tile region, so items are kept as large as that allows)
+    // work items small enough that a small species still gives every SM one, or both CTAs of every SM
+    // (each item stages a whole tile region, so items are kept as large as that allows); the plasma
+    // electrons keep to the larger items: each item rounds once on a J_z that still holds the ions'
+    // current, which theirs nearly cancels
+    const int64_t wanted = (int64_t)c->num_sms * (c->plasma && si == c->sp_e ? 1 : 2);
     s.chunk = kChunk;
-    while (s.chunk > kChunkMin && s.bound / s.chunk < (int64_t)c->num_sms) s.chunk /= 2;
+    while (s.chunk > kChunkMin && s.bound / s.chunk < wanted) s.chunk /= 2;
     TileDev t = tile_dev(c, s);
     SpeciesDev sd = species_dev(c, s);
     const int n_keys = (int)c->n_keys;

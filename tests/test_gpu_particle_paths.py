@@ -82,7 +82,7 @@ def test_hot_particles_cross_nodes(order, gather, n):
     _one_step(w, sim, ids, 9, gather)
 
 
-@pytest.mark.parametrize("tile", [(8, 8, 8), (1, 16, 5), (16, 3, 4), (5, 5, 5), (10, 8, 8)])
+@pytest.mark.parametrize("tile", [(8, 8, 8), (1, 16, 5), (16, 3, 4), (5, 5, 5), (10, 8, 8), (2, 1, 2)])
 @pytest.mark.parametrize("margin", [0, 1, 2])
 def test_tile_shapes_and_margins(tile, margin):
     # regions of other shapes (one to four CTAs per SM) and drift margins, after five steps of drift
