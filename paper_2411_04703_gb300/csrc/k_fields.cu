@@ -24,8 +24,7 @@ __device__ __forceinline__ float cpml_d(float b, float &psi, float dF)
 // Six 256-thread blocks per SM (40 registers) keep more loads in flight than four at 64; both
 // measured faster than one thread per cell, which spent ~375 instructions a cell on index and
 // face arithmetic.
-constexpr int kFdtdKzB = 8;
-constexpr int kFdtdKzE = 8;
+constexpr int kFdtdKz = 8;   // at most: see fdtd_shape
 
 // Offset of the neighbour at p + s (s = +1 or -1) of a dim of n cells with stride st: within the
 // grid the plain offset, across a periodic face the wrapped one (n = 1: the cell itself), across
@@ -84,9 +83,12 @@ __global__ void __launch_bounds__(256, 6) k_fdtd_b(const float *__restrict__ E, 
         if (pml.on) {
             const float bz = pml.bB[2][k];
             if (bx < 1.f || by < 1.f || bz < 1.f) {
-                float p[6];
-#pragma unroll
-                for (int q = 0; q < 6; q++) p[q] = psiB[q * N + ix];
+                float p[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                // (only the layers the cell is in, 2 of 6 but for edges and corners: 256 x 256 x 1024
+                // cells in layers on every face 1.97 -> 1.80 ms a step)
+                if (by < 1.f) { p[0] = psiB[0 * N + ix]; p[5] = psiB[5 * N + ix]; }
+                if (bz < 1.f) { p[1] = psiB[1 * N + ix]; p[2] = psiB[2 * N + ix]; }
+                if (bx < 1.f) { p[3] = psiB[3 * N + ix]; p[4] = psiB[4 * N + ix]; }
                 dEz_dy = cpml_d(by, p[0], dEz_dy);
                 dEy_dz = cpml_d(bz, p[1], dEy_dz);
                 dEx_dz = cpml_d(bz, p[2], dEx_dz);
@@ -154,9 +156,12 @@ __global__ void __launch_bounds__(256, 6) k_fdtd_e(float *__restrict__ E, const 
         if (pml.on) {
             const float bz = pml.bE[2][k];
             if (bx < 1.f || by < 1.f || bz < 1.f) {
-                float p[6];
-#pragma unroll
-                for (int q = 0; q < 6; q++) p[q] = psiE[q * N + ix];
+                float p[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                // (only the layers the cell is in, 2 of 6 but for edges and corners: 256 x 256 x 1024
+                // cells in layers on every face 1.97 -> 1.80 ms a step)
+                if (by < 1.f) { p[0] = psiE[0 * N + ix]; p[5] = psiE[5 * N + ix]; }
+                if (bz < 1.f) { p[1] = psiE[1 * N + ix]; p[2] = psiE[2 * N + ix]; }
+                if (bx < 1.f) { p[3] = psiE[3 * N + ix]; p[4] = psiE[4 * N + ix]; }
                 dBz_dy = cpml_d(by, p[0], dBz_dy);
                 dBy_dz = cpml_d(bz, p[1], dBy_dz);
                 dBx_dz = cpml_d(bz, p[2], dBx_dz);
@@ -247,22 +252,55 @@ __global__ void k_sumsq(const float *a, long long n, double *partial)
     }
 }
 
+// Launch shape of the two updates.  Blocks of 8 warps, each on 32 cells of x: as many rows of y as the
+// grid has, up to 8, the other warps along x (a 2-D grid has one row, and a block of 8 used one warp).
+// The walk along z is a chain of loads behind stores: a grid that does not fill the chip takes the
+// shorter walks, down to one cell a thread, that give two warps for each of the 48 an SM holds (one and
+// four measured within 2 % of it, but for a 1024 x 1 x 2048 grid: 0.083, 0.072, 0.073 ms).  A step's
+// three updates, walk of 8 against this, ms: 20 x 18 x 44 cells 0.029 / 0.015, 45 x 39 x 70 0.031 / 0.020,
+// 63 x 65 x 200 with layers 0.056 / 0.043, 1024 x 1 x 2048 0.130 / 0.072; 256 x 256 x 1024 walks 8 cells.
+struct FdtdShape {
+    dim3 grd, blk;
+    int kz;
+};
+FdtdShape fdtd_shape(const pic_ctx *c)
+{
+    int wy = 8;
+    while (wy > 1 && wy / 2 >= c->n[1]) wy /= 2;
+    const int wx = std::max(1, std::min(8 / wy, (c->n[0] + 31) / 32));
+    FdtdShape s;
+    s.blk = dim3(32 * wx, wy, 1);
+    s.grd = dim3((c->n[0] + 32 * wx - 1) / (32 * wx), (c->n[1] + wy - 1) / wy, 1);
+    const int64_t warps = (int64_t)s.grd.x * s.grd.y * wx * wy;
+    for (s.kz = kFdtdKz; s.kz > 1 && warps * ((c->n[2] + s.kz - 1) / s.kz) < 48 * (int64_t)c->num_sms * 2; ) s.kz /= 2;
+    s.grd.z = (c->n[2] + s.kz - 1) / s.kz;
+    return s;
+}
+
 }  // namespace
 
 cudaError_t launch_fdtd_b(pic_ctx *c, float dtt)
 {
-    dim3 blk(32, 8, 1), grd((c->n[0] + 31) / 32, (c->n[1] + 7) / 8, (c->n[2] + kFdtdKzB - 1) / kFdtdKzB);
+    const FdtdShape s = fdtd_shape(c);
     const PmlDev pml = pml_dev(c);
-    k_fdtd_b<kFdtdKzB><<<grd, blk, 0, c->stream>>>(c->E, c->B, pml.psiB, grid_dev(c), pml, dtt);
+    auto run = [&](auto kern) { kern<<<s.grd, s.blk, 0, c->stream>>>(c->E, c->B, pml.psiB, grid_dev(c), pml, dtt); };
+    if (s.kz == 8) run(k_fdtd_b<8>);
+    else if (s.kz == 4) run(k_fdtd_b<4>);
+    else if (s.kz == 2) run(k_fdtd_b<2>);
+    else run(k_fdtd_b<1>);
     c->kernels++;
     return cudaGetLastError();
 }
 
 cudaError_t launch_fdtd_e(pic_ctx *c)
 {
-    dim3 blk(32, 8, 1), grd((c->n[0] + 31) / 32, (c->n[1] + 7) / 8, (c->n[2] + kFdtdKzE - 1) / kFdtdKzE);
+    const FdtdShape s = fdtd_shape(c);
     const PmlDev pml = pml_dev(c);
-    k_fdtd_e<kFdtdKzE><<<grd, blk, 0, c->stream>>>(c->E, c->B, c->J, pml.psiE, grid_dev(c), pml);
+    auto run = [&](auto kern) { kern<<<s.grd, s.blk, 0, c->stream>>>(c->E, c->B, c->J, pml.psiE, grid_dev(c), pml); };
+    if (s.kz == 8) run(k_fdtd_e<8>);
+    else if (s.kz == 4) run(k_fdtd_e<4>);
+    else if (s.kz == 2) run(k_fdtd_e<2>);
+    else run(k_fdtd_e<1>);
     c->kernels++;
     return cudaGetLastError();
 }

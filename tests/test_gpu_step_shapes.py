@@ -1,0 +1,46 @@
+"""The field updates at their launch shapes against the FP64 oracle.  Tolerance: the
+repository's bar of one step, 1e-5 of the largest value per component, times the steps taken.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2411_04703_gb300 import api, workloads as W
+
+import parity
+
+pytestmark = pytest.mark.gpu
+
+TOL_STEP = 1e-5
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    oracle.build()
+
+
+# walks of 1 cell (with 1, 2, 3 and more rows of y, ragged in every dim), 2, 4 and 8 cells, the last
+# walk of a column cut short
+@pytest.mark.parametrize("grid", [(9, 1, 30), (300, 1, 21), (40, 2, 33), (5, 3, 70), (33, 7, 41),
+                                  (33, 64, 233), (33, 64, 461), (33, 64, 919)])
+@pytest.mark.parametrize("layers", [False, True])
+def test_field_update_shapes(grid, layers):
+    d, dt = (0.5, 0.6, 0.55), 0.27
+    face = [(W.PML, W.PML) if layers and n >= 20 else (W.PERIODIC, W.PERIODIC) for n in grid]
+    sim = api.Sim(grid, d, dt, 1.0, bc=face, pml=6 if layers else 0)
+    o = oracle.Sim(grid, d, dt, 1.0, bc=face, pml=6 if layers else 0)
+    rng = np.random.default_rng(sum(grid))
+    for c in range(6):
+        f = rng.standard_normal((grid[2], grid[1], grid[0])).astype(np.float32)
+        sim.set_field(c, f)
+        o.set_field(c, f.astype(np.float64))
+    steps = 2                                   # the second meets the layers' psi of the first
+    sim.step(steps)
+    sim.sync()
+    for _ in range(steps):
+        o.fdtd()
+    f = parity.compare_fields(sim, o, range(6))
+    assert max(f.values()) < steps * TOL_STEP, f
