@@ -886,8 +886,6 @@ int pic_set_plasma_batch(pic_ctx *c, const pic_plasma *p, const double *density_
 
 namespace {
 
-__global__ void k_tick(long long *clock) { *clock += 1; }
-
 int save_state(pic_ctx *c, StateSnap &st, bool alloc, bool quick = false);
 int ad_checkpoint_due(pic_ctx *c);
 
@@ -914,7 +912,6 @@ int step_once(pic_ctx *c)
     // the lattice species writes J_z whole, before the other species add to it
     const bool lat = c->plasma && c->sp[c->sp_i].lattice;
     CK(cudaMemsetAsync(c->J, 0, sizeof(float) * (lat ? 2 : 3) * c->ncell, c->stream));
-    CK(cudaMemsetAsync(c->work, 0, sizeof(int) * 2 * kMaxSpecies, c->stream));
     if (lat) {
         TraceScope ts(c, TR_PUSH_FROZEN);
         CK(launch_lattice_step(c, c->sp_i));
@@ -944,9 +941,7 @@ int step_once(pic_ctx *c)
         CK(launch_fdtd_e(c));
         CK(launch_fdtd_b(c, (float)(0.5 * c->dt)));
     }
-    k_tick<<<1, 1, 0, c->stream>>>(c->dclock);
-    CK(cudaGetLastError());
-    c->kernels++;
+    CK(launch_step_end(c));
     c->step++;
     if (c->moving) {
         const int64_t due = (int64_t)shifts_due(c, c->step);

@@ -324,6 +324,7 @@ PmlDev pml_dev(const pic_ctx *c);
 // k_push.cu
 cudaError_t launch_push(pic_ctx *c, int si, const ExtDev &ext);
 cudaError_t launch_dlim_from_momenta(pic_ctx *c, int si);
+cudaError_t launch_step_end(pic_ctx *c);   // displacement bounds, clock and work counters
 cudaError_t launch_rho(pic_ctx *c, const Species &s, float *rho);
 // k_lattice.cu
 cudaError_t launch_lattice_profiles(pic_ctx *c, int si);

@@ -77,7 +77,46 @@ __global__ void k_dmax_measure(SpeciesDev sp, float tx, float ty, float tz)
     }
 }
 
+// The end of a step in one launch (a dependent launch costs a small grid 2-3 us): the displacement
+// bounds of the species pushed, the clock, and the particle kernels' work counters back to zero for the
+// next step.
+struct StepEnd {
+    long long *clock;
+    int *work;
+    float *dlim[kMaxSpecies];
+    unsigned *dmax[kMaxSpecies];
+    float light[3];
+    int n;
+};
+__global__ void k_step_end(StepEnd e)
+{
+    const int q = threadIdx.x, s = q / 3, k = q % 3;
+    if (s < e.n) push::dlim_update(e.dlim[s], e.dmax[s], k, k == 0 ? e.light[0] : (k == 1 ? e.light[1] : e.light[2]));
+    if (q < 2 * kMaxSpecies && e.work) e.work[q] = 0;
+    if (q == 0 && e.clock) *e.clock += 1;
+}
+
+void add_dlim(StepEnd &e, const pic_ctx *c, const Species &s)
+{
+    for (int d = 0; d < 3; d++) e.light[d] = (float)std::min(1.0, c->dt / c->d[d]);
+    e.dlim[e.n] = s.dlim;
+    e.dmax[e.n++] = s.dmax;
+}
+
 }  // namespace
+
+cudaError_t launch_step_end(pic_ctx *c)
+{
+    static_assert(3 * kMaxSpecies <= 32, "a thread per component of a species");
+    StepEnd e{};
+    e.clock = c->dclock;
+    e.work = c->work;
+    for (int si = 0; si < c->nsp; si++)
+        if (!c->sp[si].lattice) add_dlim(e, c, c->sp[si]);
+    k_step_end<<<1, 32, 0, c->stream>>>(e);
+    c->kernels++;
+    return cudaGetLastError();
+}
 
 // Sets the displacement bound of species si from its current momenta (after a load or an
 // injection): four times the largest displacement they give, as after a step.
@@ -85,13 +124,13 @@ cudaError_t launch_dlim_from_momenta(pic_ctx *c, int si)
 {
     const Species &s = c->sp[si];
     if (s.lattice || !s.dlim) return cudaSuccess;
-    float light[3];
-    for (int d = 0; d < 3; d++) light[d] = (float)std::min(1.0, c->dt / c->d[d]);
     k_dmax_measure<<<c->num_sms * 4, 256, 0, c->stream>>>(species_dev(c, s), (float)(c->dt / c->d[0]),
                                                           (float)(c->dt / c->d[1]), (float)(c->dt / c->d[2]));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    push::k_dlim_update<<<1, 32, 0, c->stream>>>(s.dlim, s.dmax, light[0], light[1], light[2]);
+    StepEnd u{};
+    add_dlim(u, c, s);
+    k_step_end<<<1, 32, 0, c->stream>>>(u);
     c->kernels += 2;
     return cudaGetLastError();
 }

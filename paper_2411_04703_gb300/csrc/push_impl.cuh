@@ -822,11 +822,8 @@ k_push_frozen(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int
 
 // Next step's displacement bound per component: four times the largest displacement of this step,
 // within [light * 2^-10, light] (light: the speed-of-light bound); the measurement restarts.
-static __global__ void k_dlim_update(float *dlim, unsigned *dmax, float l0, float l1, float l2)
+__device__ __forceinline__ void dlim_update(float *dlim, unsigned *dmax, int k, float light)
 {
-    const int k = threadIdx.x;
-    if (k >= 3) return;
-    const float light = k == 0 ? l0 : (k == 1 ? l1 : l2);
     const float m = __uint_as_float(dmax[k]);
     dlim[k] = fminf(light, fmaxf(4.f * m, light * 0x1p-10f));
     dmax[k] = 0u;
@@ -864,15 +861,6 @@ struct KernelCache {
     }
 };
 
-inline cudaError_t launch_dlim_update(pic_ctx *c, const Species &s)
-{
-    float light[3];
-    for (int d = 0; d < 3; d++) light[d] = (float)std::min(1.0, c->dt / c->d[d]);
-    k_dlim_update<<<1, 32, 0, c->stream>>>(s.dlim, s.dmax, light[0], light[1], light[2]);
-    c->kernels += 2;   // with the particle kernel before it
-    return cudaGetLastError();
-}
-
 // Compile-time region for the default tile (8^3 cells, drift margin 1); any other tuning uses
 // the runtime-sized region.
 inline bool default_region(const pic_ctx *c)
@@ -893,8 +881,8 @@ cudaError_t launch_frozen_t(pic_ctx *c, int si, const ExtDev &ext, Reg reg, int 
     kern<<<c->num_sms * per_sm, kPushThreads, smem, c->stream>>>(species_dev(c, s), grid_dev(c), tile_dev(c, s),
                                                                   FieldsDev{c->E, c->B, c->J}, ext, c->work + si,
                                                                   c->work + kMaxSpecies + si, c->err, reg);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return launch_dlim_update(c, s);
+    c->kernels++;
+    return cudaGetLastError();
 }
 
 // Frozen species: the region spans the tile, its drift margin and the general deposit window.

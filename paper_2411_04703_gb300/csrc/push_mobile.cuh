@@ -454,8 +454,8 @@ cudaError_t launch_push_t(pic_ctx *c, int si, const ExtDev &ext, Reg reg, int R3
     if (e != cudaSuccess) return e;
     kern<<<c->num_sms * std::min(per_sm, MINB), NT, smem, c->stream>>>(species_dev(c, s), grid_dev(c), tile_dev(c, s), FieldsDev{c->E, c->B, c->J},
                                                         ext, c->work + si, c->work + kMaxSpecies + si, c->err, reg, sort_age(c));
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return launch_dlim_update(c, s);
+    c->kernels++;
+    return cudaGetLastError();
 }
 
 // The region of a tile: its cells and drift margin, one node below and (TSC) two or (CIC) one above.

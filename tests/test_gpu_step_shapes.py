@@ -1,4 +1,4 @@
-"""The field updates at their launch shapes against the FP64 oracle.  Tolerance: the
+"""The field updates' launch shapes and the end of a step against the FP64 oracle.  Tolerance: the
 repository's bar of one step, 1e-5 of the largest value per component, times the steps taken.
 """
 import numpy as np
@@ -43,4 +43,32 @@ def test_field_update_shapes(grid, layers):
     for _ in range(steps):
         o.fdtd()
     f = parity.compare_fields(sim, o, range(6))
+    assert max(f.values()) < steps * TOL_STEP, f
+
+
+@pytest.mark.parametrize("n_species", [1, 3, 8])
+def test_step_end_serves_every_species(n_species):
+    # each species has its own bound on a step's displacement, its own counters and the common clock
+    w = W.vacuum_undulator(grid=(20, 10, 18), n_beam=900, seed=3, order=2)
+    sim, _ = api.from_workload(w, beam=False)
+    o, oid = parity.oracle_from_gpu(w, sim, {})
+    ids = []
+    for s in range(n_species):
+        X, U, Wt = W.sample_uniform_particles(w.grid, 900, seed=50 + s, umax=0.02 * 2.0 ** s)
+        ids.append(sim.load_species(-1.0, 1.0, X.T * np.array(w.d)[:, None], U.T, Wt * 1e-3, frame=api.PIC_FRAME_BOOSTED))
+        P = sim.get_particles(ids[s])
+        oid[s] = o.add_species(-1.0, 1.0, capacity=1024)
+        o.set_state(oid[s], P["cell"].astype(np.float64) + P["off"].astype(np.float64), P["u"].astype(np.float64),
+                    P["w"].astype(np.float64), P["id"])
+    steps = 3
+    sim.step(steps)
+    sim.sync()
+    o.step(steps)
+    assert sim.get_time()[0] == steps
+    w.beam.q, w.beam.m = -1.0, 1.0
+    for s in range(n_species):
+        r = parity.compare_species(w, sim, ids[s], o, oid[s])
+        assert r["only_gpu"] == 0 and r["only_oracle"] == 0, (s, r)
+        assert r["u_rel_err"] < steps * TOL_STEP and r["pos_abs_err"] < steps * 1e-5, (s, r)
+    f = parity.compare_fields(sim, o)
     assert max(f.values()) < steps * TOL_STEP, f
