@@ -234,8 +234,11 @@ __global__ void k_shift_fields(float *const *arrays, int n_arrays, int nx, int n
     A[(long long)(nz - 1) * plane + col] = 0.f;
 }
 
-__global__ void k_sumsq(const float *a, long long n, double *partial)
+// Sums of squares of n values of each of the six field components (blockIdx.y), a partial sum a block.
+__global__ void k_sumsq(const float *E, const float *B, long long ncell, long long n, double *partial)
 {
+    const int q = blockIdx.y;
+    const float *a = q < 3 ? E + q * ncell : B + (q - 3) * ncell;
     double s = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const double v = a[i];
@@ -248,9 +251,10 @@ __global__ void k_sumsq(const float *a, long long n, double *partial)
     if (threadIdx.x < 32) {
         s = threadIdx.x < (blockDim.x >> 5) ? ws[threadIdx.x] : 0.0;
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) partial[blockIdx.x] = s;
+        if (threadIdx.x == 0) partial[q * gridDim.x + blockIdx.x] = s;
     }
 }
+
 
 // Launch shape of the two updates.  Blocks of 8 warps, each on 32 cells of x: as many rows of y as the
 // grid has, up to 8, the other warps along x (a 2-D grid has one row, and a block of 8 used one warp).
@@ -341,24 +345,22 @@ cudaError_t launch_shift_fields(pic_ctx *c)
 // (1/2) sum (E^2 + B^2) dV over the grid, or over the rows of one run of an ensemble (run >= 0).
 cudaError_t launch_field_energy(pic_ctx *c, double *out_host, int run)
 {
+    // one launch and one read for the six components (a read of each waited six times for the device)
     const int blocks = 1024;
-    double acc = 0.0;
-    std::vector<double> part(blocks);
+    std::vector<double> part(6 * blocks);
     const long long plane = (long long)c->n[0] * c->n[1];
     const long long off = run < 0 ? 0 : (long long)run * c->nzr * plane;
     const long long len = run < 0 ? c->ncell : (long long)c->nzr * plane;
-    for (int q = 0; q < 6; q++) {
-        const float *a = (q < 3 ? c->E + q * c->ncell : c->B + (q - 3) * c->ncell) + off;
-        k_sumsq<<<blocks, 256, 0, c->stream>>>(a, len, c->red);
-        c->kernels++;
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        e = cudaMemcpyAsync(part.data(), c->red, blocks * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-        if (e != cudaSuccess) return e;
-        e = cudaStreamSynchronize(c->stream);
-        if (e != cudaSuccess) return e;
-        for (int b = 0; b < blocks; b++) acc += part[b];
-    }
+    k_sumsq<<<dim3(blocks, 6), 256, 0, c->stream>>>(c->E + off, c->B + off, c->ncell, len, c->red);
+    c->kernels++;
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpyAsync(part.data(), c->red, part.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+    if (e != cudaSuccess) return e;
+    e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return e;
+    double acc = 0.0;
+    for (double v : part) acc += v;
     *out_host = 0.5 * acc * c->d[0] * c->d[1] * c->d[2];
     return cudaSuccess;
 }
