@@ -24,6 +24,10 @@ namespace gbpic {
 namespace {
 
 constexpr int kAdjThreads = 256;
+// Keys a warp sums per group, and the lanes from which a group pays for its 48 shuffles.  Reverse sweep of
+// 20 steps on 64 x 64 x 256 cells, 2M beam: whole warps of one key only 66.0 ms a gradient, 3 groups of 4
+// lanes 57.9, 6 of 4 57.2, 6 of 8 57.6, 10 of 3 57.8.
+constexpr int kAdjGroups = 6, kAdjGroup = 4;
 
 __device__ __forceinline__ int wrapi(int i, int n) { return pwrap(i, n); }
 
@@ -354,20 +358,31 @@ __global__ void __launch_bounds__(kAdjThreads, 2) k_adj_particles(AdjP a)
         // ---- adjoint of the gather and the external field
         const float lF[6] = {live ? lE[0] : 0.f, live ? lE[1] : 0.f, live ? lE[2] : 0.f,
                              live ? lB[0] : 0.f, live ? lB[1] : 0.f, live ? lB[2] : 0.f};
-        // The 48 scatter targets follow from the cell and the staggered-window choice.  Where
-        // all 32 lanes of the warp share both (the core of a dense beam, ~1000 particles per
-        // cell, sorted by cell and octant), the warp sums the 48 values by a transpose
-        // reduction: each exchange halves the values a lane holds (24, 12, 6, 3 for lane bits
-        // 4..1; the last pair swaps all three), 48 shuffles in all; lane L ends with the totals
-        // of value indices 3 (L >> 1) .. 3 (L >> 1) + 2 and issues one or two atomics.  Other
-        // warps scatter their own values, 48 atomics per particle.
-        const long long key = live ? (((long long)cell << 3) | oct) : -1ll - (long long)lane;
-        const bool uniform = __all_sync(0xffffffffu, key == __shfl_sync(0xffffffffu, key, 0));
+        // The 48 scatter targets follow from the cell and the staggered-window choice (the key).  Lanes
+        // of a warp that share both (a dense beam, ~1000 particles per cell, sorted by cell and octant;
+        // since the sort it has drifted over a few keys) are summed by a transpose reduction in which
+        // the other lanes hold zeros: each exchange halves the values a lane holds (24, 12, 6, 3 for
+        // lane bits 4..1; the last pair swaps all three), 48 shuffles in all; lane L ends with the
+        // totals of value indices 3 (L >> 1) .. 3 (L >> 1) + 2 and issues one or two atomics.  At most
+        // kAdjGroups keys a warp, of kAdjGroup lanes or more; the other lanes scatter their own values,
+        // 48 atomics a particle.
+        const long long key = live ? (((long long)cell << 3) | oct) : -1ll;
 #pragma unroll
         for (int comp = 0; comp < 6; comp++)
 #pragma unroll
             for (int d = 0; d < 3; d++) lo[d] = fmaf(lF[comp], dF[comp][d], lo[d]);
-        if (uniform) {
+        bool own = live;                  // it scatters its own values
+        unsigned todo = __ballot_sync(0xffffffffu, live);
+        for (int group = 0; group < kAdjGroups && todo; group++) {
+            const int src = __ffs(todo) - 1;
+            const long long gkey = __shfl_sync(0xffffffffu, key, src);
+            const bool mine = key == gkey;
+            const unsigned members = __ballot_sync(0xffffffffu, mine);
+            todo &= ~members;
+            if (__popc(members) < kAdjGroup) continue;
+            own = own && !mine;
+            const int gcell = (int)(gkey >> 3), goct = (int)(gkey & 7);
+            const int gc[3] = {g.cc.i(gcell), g.cc.j(gcell), g.cc.k(gcell)};
             // value index vi = comp * 8 + k * 4 + j * 2 + i: its weight, then its node
             auto val = [&](int vi) {
                 const int comp = vi >> 3, i = vi & 1, j = (vi >> 1) & 1, k = (vi >> 2) & 1;
@@ -377,7 +392,7 @@ __global__ void __launch_bounds__(kAdjThreads, 2) k_adj_particles(AdjP a)
                 const float wx = st0 ? ws[0][i] : wu[0][i];
                 const float wy = st1 ? ws[1][j] : wu[1][j];
                 const float wz = st2 ? ws[2][k] : wu[2][k];
-                return wx * wy * wz * lF[comp];
+                return mine ? wx * wy * wz * lF[comp] : 0.f;
             };
             float h24[24], h12[12], h6[6], h3[3];
             const bool b4 = lane & 16u, b3 = lane & 8u, b2 = lane & 4u, b1 = lane & 2u;
@@ -408,14 +423,15 @@ __global__ void __launch_bounds__(kAdjThreads, 2) k_adj_particles(AdjP a)
 #pragma unroll
                     for (int d = 0; d < 3; d++) {
                         const bool st = comp < 3 ? comp == d : comp - 3 != d;
-                        const int x = wrapi(c[d] + qq[d] - ((st && ((oct >> d) & 1)) ? 1 : 0), g.n[d]);
+                        const int x = wrapi(gc[d] + qq[d] - ((st && ((goct >> d) & 1)) ? 1 : 0), g.n[d]);
                         ix += d == 0 ? x : (d == 1 ? x * g.n[0] : x * g.n[0] * g.n[1]);
                     }
                     float *lf = comp < 3 ? a.lE + comp * g.ncell : a.lB + (comp - 3) * g.ncell;
                     atomicAdd(lf + ix, h3[q]);
                 }
             }
-        } else {
+        }
+        if (own) {
 #pragma unroll
             for (int comp = 0; comp < 6; comp++) {
                 const bool st0 = comp < 3 ? comp == 0 : comp != 3;

@@ -119,3 +119,21 @@ def test_adjoint_matches_gpu_central_differences(adjoint):
     assert g["dL_dK"] == pytest.approx(dK, rel=3e-2), (g["dL_dK"], dK)
     # (the profile's effect on the loss, ~1e-7 per node, is below the FP32 forward's rounding at
     # h = 1e-4; the oracle's FP64 differences check that part)
+
+
+# Beams a few cells wide, whose warps share scatter windows in groups of 1 to 32 lanes; the checkpoints
+# between the sorts let the groups drift apart.  Tolerance: that of the wider beam above.
+@pytest.mark.parametrize("squeeze, every", [(0.4, 10), (0.2, 3)])
+def test_adjoint_of_a_dense_beam_matches_fp64_oracle(squeeze, every):
+    w = _workload()
+    w.steps = 10
+    w.beam.sigma_r *= squeeze
+    sim, ids = api.from_workload(w)
+    sim.checkpoint(every)
+    sim.step(w.steps)
+    g = sim.backward(ids["beam"], _k_rrf(w))
+    sim.close()
+    K0 = w.undulator.K
+    dK = (_oracle_loss(w, K0 * (1 + H)) - _oracle_loss(w, K0 * (1 - H))) / (2 * H * K0)
+    assert g["loss"] == pytest.approx(_oracle_loss(w), rel=1e-4)
+    assert g["dL_dK"] == pytest.approx(dK, rel=2e-3), (g["dL_dK"], dK)
