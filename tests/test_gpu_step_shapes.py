@@ -72,3 +72,26 @@ def test_step_end_serves_every_species(n_species):
         assert r["u_rel_err"] < steps * TOL_STEP and r["pos_abs_err"] < steps * 1e-5, (s, r)
     f = parity.compare_fields(sim, o)
     assert max(f.values()) < steps * TOL_STEP, f
+
+
+# One particle, a cold pair, a hot cloud: the two passes' shift about the mean particle.  FP64 on the
+# same records: 1e-9 of a value; a spread also within 1e-7 of the largest coordinate, ten times the root
+# of FP64 rounding (a single particle has none).
+@pytest.mark.parametrize("n, umax", [(1, 0.5), (2, 0.0), (3000, 4.0)])
+@pytest.mark.parametrize("frame, oframe", [(api.PIC_FRAME_LAB, 1), (api.PIC_FRAME_BOOSTED, 0)])
+def test_moments_in_two_passes(n, umax, frame, oframe):
+    w = W.vacuum_undulator(grid=(20, 10, 18), n_beam=n, seed=3, order=2)
+    sim, _ = api.from_workload(w, beam=False)
+    o, _ = parity.oracle_from_gpu(w, sim, {})
+    X, U, Wt = W.sample_uniform_particles(w.grid, n, seed=70 + n, umax=umax)
+    sid = sim.load_species(-1.0, 1.0, X.T * np.array(w.d)[:, None], U.T, Wt, frame=api.PIC_FRAME_BOOSTED)
+    P = sim.get_particles(sid)
+    s = o.add_species(-1.0, 1.0, capacity=max(n, 1))
+    o.set_state(s, P["cell"].astype(np.float64) + P["off"].astype(np.float64), P["u"].astype(np.float64),
+                P["w"].astype(np.float64), P["id"])
+    g, r = sim.get_moments(sid, frame, k_bunch=3.0), o.moments(s, frame=oframe, k=3.0)
+    scale = max(abs(r[k]) for k in ("mean_x", "mean_y", "mean_z", "mean_gamma"))
+    for k in ("count", "mean_x", "mean_y", "mean_z", "mean_uz", "mean_gamma", "bunching", "kinetic_energy", "mean_t"):
+        assert g[k] == pytest.approx(r[k], rel=1e-9, abs=1e-12), (k, g[k], r[k])
+    for k in ("rms_x", "rms_y", "rms_z", "rel_energy_spread", "emit_nx", "emit_ny"):
+        assert g[k] == pytest.approx(r[k], rel=1e-9, abs=1e-7 * scale), (k, g[k], r[k])
