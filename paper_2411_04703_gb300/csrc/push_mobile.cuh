@@ -126,7 +126,7 @@ __device__ __forceinline__ void deposit_cross(const SmemAcc<Reg> &acc, const flo
 //    0.330 -> 0.320).
 // ms per step, with the cell-ordered lanes -> one CTA of 512 threads -> two CTAs: plasma buncher
 // 5.22 -> 4.15 -> 3.80, sweep of 64 runs 18.0 -> 15.1 -> 13.6, long undulator 4.66 -> 4.19 -> 4.12, 65k
-// electrons CIC 0.045 -> 0.046 -> 0.033 (the region follows the drift), 2-D buncher 2.40 -> 1.40 -> 1.21.
+// electrons CIC 0.045 -> 0.046 -> 0.033 (the region follows the drift), 2-D buncher 2.40 -> 1.40 (1.76 with one CTA: launch_push_dyn).
 template <int ORDER, int GATHER, int NT, int MINB, class Reg>
 __global__ void __launch_bounds__(NT, MINB)
 k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work, int *work_sparse, int *err, Reg reg, int age)
