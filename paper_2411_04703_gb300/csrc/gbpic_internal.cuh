@@ -315,6 +315,17 @@ struct pic_ctx {
 
 namespace gbpic {
 
+// Whether species si's current is nearly cancelled by another one's, so that the fields are driven by a
+// small difference in which the rounding of every addition shows: the electrons of a plasma (its ions'
+// current is written first), or, of species loaded one by one, those with another of the opposite charge.
+inline bool cancels(const pic_ctx *c, int si)
+{
+    if (c->plasma) return si == c->sp_e;
+    for (int q = 0; q < c->nsp; q++)
+        if (c->sp[q].q * c->sp[si].q < 0.0) return true;
+    return false;
+}
+
 GridDev grid_dev(const pic_ctx *c);
 TileDev tile_dev(const pic_ctx *c, const Species &s);
 SpeciesDev species_dev(const pic_ctx *c, const Species &s);

@@ -276,7 +276,7 @@ cudaError_t launch_sort(pic_ctx *c, int si, bool by_octant)
     // (each item stages a whole tile region, so items are kept as large as that allows); the plasma
     // electrons keep to the larger items: each item rounds once on a J_z that still holds the ions'
     // current, which theirs nearly cancels
-    const int64_t wanted = (int64_t)c->num_sms * (c->plasma && si == c->sp_e ? 1 : 2);
+    const int64_t wanted = (int64_t)c->num_sms * (cancels(c, si) ? 1 : 2);
     s.chunk = kChunk;
     while (s.chunk > kChunkMin && s.bound / s.chunk < wanted) s.chunk /= 2;
     TileDev t = tile_dev(c, s);

@@ -63,6 +63,10 @@ template <int RX, int RY, int RZ, int R2 = plane_pitch(RX, RY)> struct RegFix {
 // piece, so piece = length * S'(midpoint) is exact, and the length before the knot is taken in
 // offset space, (m + k) - o, which is exact near a crossing.  A slow component (|d| << 1 cell)
 // thus keeps full FP32 relative precision in its current.
+// The length behind the knot, d - a, is taken from the product v h that d rounds (one rounding); with
+// (v, h) = (d, 1) it is taken from the rounded displacement.  A cold lattice crosses all at once and
+// rounds alike, and a neutral plasma's current is a small difference of large ones, so this last digit
+// is visible in its fields (1e-3 of E): the callers spell out which of the two they take.
 template <int ORDER> struct Shape;
 
 // Order 0 (nearest grid point), used only by the energy-conserving gather of the first-order
@@ -90,20 +94,22 @@ template <> struct Shape<1> {
     __device__ __forceinline__ static float dS(float t) {
         return fabsf(t) < 1.f ? (t > 0.f ? -1.f : (t < 0.f ? 1.f : 0.f)) : 0.f;
     }
-    __device__ __forceinline__ static float seg(float o, int m, float d) {
+    __device__ __forceinline__ static float seg(float o, int m, float d, float v, float h) {
         const float t0 = o - (float)m, t1 = t0 + d;
         const float lo = fminf(t0, t1), hi = fmaxf(t0, t1);
         const float k = ceilf(hi) - 1.f;            // largest knot below hi
         if (!(k > lo)) return d * dS(t0 + 0.5f * d);
         const float a = ((float)m + k) - o;
-        return a * dS(k - 0.5f * a) + (d - a) * dS(k + 0.5f * (d - a));
+        const float b = fmaf(v, h, -a);
+        return fmaf(a, dS(k - 0.5f * a), __fmul_rn(b, dS(k + 0.5f * b)));
     }
-    __device__ __forceinline__ static void general(float o, float d, int s, int &st, float S0[3], float DS[3]) {
+    __device__ __forceinline__ static void general(float o, float d, int s, float v, float h, int &st, float S0[3],
+                                                   float DS[3]) {
         st = min(s, 0);
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             S0[a] = S(o - (float)(st + a));
-            DS[a] = seg(o, st + a, d);
+            DS[a] = seg(o, st + a, d, v, h);
         }
     }
     // the cell does not change: window {c, c+1}
@@ -138,22 +144,24 @@ template <> struct Shape<2> {
         const float v = a <= 0.5f ? -2.f * a : (a < 1.5f ? a - 1.5f : 0.f);
         return t < 0.f ? -v : v;
     }
-    __device__ __forceinline__ static float seg(float o, int m, float d) {
+    __device__ __forceinline__ static float seg(float o, int m, float d, float v, float h) {
         const float t0 = o - (float)m, t1 = t0 + d;
         const float lo = fminf(t0, t1), hi = fmaxf(t0, t1);
         const float k = ceilf(hi - 0.5f) - 0.5f;    // largest knot below hi
         if (!(k > lo)) return d * dS(t0 + 0.5f * d);
         const float a = ((float)m + k) - o;
-        return a * dS(k - 0.5f * a) + (d - a) * dS(k + 0.5f * (d - a));
+        const float b = fmaf(v, h, -a);
+        return fmaf(a, dS(k - 0.5f * a), __fmul_rn(b, dS(k + 0.5f * b)));
     }
-    __device__ __forceinline__ static void general(float o, float d, int /*s*/, int &st, float S0[4], float DS[4]) {
+    __device__ __forceinline__ static void general(float o, float d, int /*s*/, float v, float h, int &st, float S0[4],
+                                                   float DS[4]) {
         const int b0 = o >= 0.5f;
         const int b1 = (int)floorf(o + d + 0.5f);   // nearest node of the new position, rel. to c
         st = b0 - 1 + min(b1 - b0, 0);
 #pragma unroll
         for (int a = 0; a < 4; a++) {
             S0[a] = S(o - (float)(st + a));
-            DS[a] = seg(o, st + a, d);
+            DS[a] = seg(o, st + a, d, v, h);
         }
     }
     // the nearest node does not change: window {b-1, b, b+1}; with dl = o - b in [-1/2, 1/2),
@@ -374,18 +382,25 @@ __device__ __forceinline__ void esirkepov(Acc &acc, const int st[3], const float
         }
 }
 
-// General window (order+2 nodes per dim), any move below one cell.
+// General window (order+2 nodes per dim), any move below one cell; d the rounded v h (see Shape).
 template <int ORDER, class Acc>
-__device__ __forceinline__ void deposit_general(Acc &acc, const float o[3], const float d[3],
-                                                const int s[3], const float fac[3])
+__device__ __forceinline__ void deposit_general(Acc &acc, const float o[3], const float d[3], const int s[3],
+                                                const float fac[3], const float v[3], const float h[3])
 {
     using S = Shape<ORDER>;
     constexpr int L = S::L;
     int st[3];
     float S0[3][L], DS[3][L];
 #pragma unroll
-    for (int dd = 0; dd < 3; dd++) S::general(o[dd], d[dd], s[dd], st[dd], S0[dd], DS[dd]);
+    for (int dd = 0; dd < 3; dd++) S::general(o[dd], d[dd], s[dd], v[dd], h[dd], st[dd], S0[dd], DS[dd]);
     esirkepov<L, true>(acc, st, S0, DS, fac, d[0] == 0.f, d[1] == 0.f);
+}
+
+template <int ORDER, class Acc>
+__device__ __forceinline__ void deposit_general(Acc &acc, const float o[3], const float d[3], const int s[3], const float fac[3])
+{
+    const float one[3] = {1.f, 1.f, 1.f};
+    deposit_general<ORDER>(acc, o, d, s, fac, d, one);
 }
 
 // Nearest node / cell unchanged in every dimension: window of order+1 nodes.
@@ -492,11 +507,11 @@ __device__ __forceinline__ void push_u(Acc &acc, const float o[3], const int c[3
     kick(o, c, E, B, mo, sp, ext);
 }
 
-// Move of one particle: d the displacement (cells), s the cell shift, o1 the new offsets and c the
-// new cell.  False when the particle left through a non-periodic face or its momentum is not finite
+// Move of one particle: v the velocity, d the displacement (cells), s the cell shift, o1 the new
+// offsets and c the new cell.  False when the particle left through a non-periodic face or its momentum is not finite
 // (it becomes a dummy).
 __device__ __forceinline__ bool move(const float o[3], int c[3], const float4 &mo, const GridDev &g, int *err, float d[3],
-                                     int s[3], float o1[3], int zb)
+                                     int s[3], float o1[3], int zb, float v[3])
 {
     const float u[3] = {mo.x, mo.y, mo.z};
     const float ig = rsqrtf(1.f + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
@@ -507,9 +522,9 @@ __device__ __forceinline__ bool move(const float o[3], int c[3], const float4 &m
         // the displacement of the push (cells), and the new offset with one rounding; both are spelt
         // out, so that every path (and build) moves a particle to the same place: a cold lattice's
         // particles round alike, and a neutral plasma's current is a small difference of large ones
-        const float v = __fmul_rn(u[dd], ig);
-        d[dd] = __fmul_rn(v, g.dt_over_d[dd]);
-        const float x1 = fmaf(v, g.dt_over_d[dd], o[dd]);
+        v[dd] = __fmul_rn(u[dd], ig);
+        d[dd] = __fmul_rn(v[dd], g.dt_over_d[dd]);
+        const float x1 = fmaf(v[dd], g.dt_over_d[dd], o[dd]);
         s[dd] = (int)floorf(x1);
         o1[dd] = x1 - (float)s[dd];
         if (o1[dd] >= 1.f) { o1[dd] = 0.f; s[dd] += 1; }
@@ -529,10 +544,10 @@ __device__ __forceinline__ bool move(const float o[3], int c[3], const float4 &m
 template <int ORDER, bool FROZEN, class Acc, int GATHER = 0>
 __device__ __forceinline__ bool push_move(Acc &acc, const float o[3], int c[3], float4 &mo,
                                           const SpeciesDev &sp, const GridDev &g, const ExtDev &ext,
-                                          int *err, float d[3], int s[3], float o1[3], int zb)
+                                          int *err, float d[3], int s[3], float o1[3], int zb, float v[3])
 {
     if (!FROZEN) push_u<ORDER, Acc, GATHER>(acc, o, c, mo, sp, ext);
-    return move(o, c, mo, g, err, d, s, o1, zb);
+    return move(o, c, mo, g, err, d, s, o1, zb, v);
 }
 
 // First node of the general deposit window, relative to the cell.
@@ -561,11 +576,14 @@ __device__ __forceinline__ void step_record(float4 &P, float4 &mo, const Species
     const float o[3] = {P.x, P.y, P.z};
     const int zb = g.nzr == g.n[2] ? 0 : zblock(c[2], g.nzr);
     GlobAcc<ORDER> acc(f, g, c, err, zb);
-    float d[3], o1[3];
+    float d[3], o1[3], v[3];
     int s[3];
-    if (push_move<ORDER, FROZEN, GlobAcc<ORDER>, GATHER>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb)) {
+    if (push_move<ORDER, FROZEN, GlobAcc<ORDER>, GATHER>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb, v)) {
         const float fac[3] = {sp.cf[0] * mo.w, sp.cf[1] * mo.w, sp.cf[2] * mo.w};
-        deposit_general<ORDER>(acc, o, d, s, fac);
+        // (TSC, along z: from the product, see Shape)
+        const bool product = ORDER == 2 && !FROZEN;
+        const float vz[3] = {d[0], d[1], product ? v[2] : d[2]}, hz[3] = {1.f, 1.f, product ? g.dt_over_d[2] : 1.f};
+        deposit_general<ORDER>(acc, o, d, s, fac, vz, hz);
         P = make_float4(o1[0], o1[1], o1[2], __int_as_float(g.cc.pack(c[0], c[1], c[2])));
         if (dmax)
 #pragma unroll
@@ -722,9 +740,9 @@ k_push_frozen(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int
             const float o[3] = {P.x, P.y, P.z};
             const int base = (rel[2] + t.M + t.hl) * reg.r2() + (rel[1] + t.M + t.hl) * Rx + rel[0] + t.M + t.hl;
             SmemAcc<Reg> acc{reg, nullptr, sJlo, sJhi, s_js, base};
-            float d[3], o1[3];
+            float d[3], o1[3], v[3];
             int s[3];
-            if (push_move<ORDER, true, SmemAcc<Reg>>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb)) {
+            if (push_move<ORDER, true, SmemAcc<Reg>>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb, v)) {
                 const float fac[3] = {sp.cf[0] * mo.w, sp.cf[1] * mo.w, sp.cf[2] * mo.w};
 #pragma unroll
                 for (int k = 0; k < 3; k++) dm[k] = __float_as_uint(fabsf(d[k]));

@@ -18,7 +18,7 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Shape values and differences on the simple window by the general window's formulas: what
-// deposit_general forms at these nodes, bit by bit (its other nodes are empty while the nearest node
+// deposit_general forms at these nodes, bit by bit (beyond them it holds zeros while the nearest node
 // stays).  A cold lattice crosses all at once and rounds alike, and its electrons' and ions' currents
 // nearly cancel: a crossing particle's current keeps the form it has on every other path (2 % of the
 // kernel where a quarter of the particles cross).
@@ -30,32 +30,34 @@ __device__ __forceinline__ void shapes_general(float o, float d, int &st, float 
 #pragma unroll
     for (int a = 0; a <= ORDER; a++) {
         S0[a] = S::S(o - (float)(st + a));
-        DS[a] = S::seg(o, st + a, d);
+        DS[a] = S::seg(o, st + a, d, d, 1.f);
     }
 }
 
 // Deposit of a particle whose nearest node (TSC) or cell (CIC) changes along one dim only (e): the
 // window is a node longer along e than the simple one and as long along the two others, 75 nodes for
 // TSC against the general window's 144 and without the general window's tests at every node.  The
-// dims are taken in the cyclic order e, e + 1, e + 2 with their strides, so one code serves all.
+// dims are taken in the cyclic order e, e + 1, e + 2 with their strides, so one code serves all.  The
+// prefix over the simple window's last node is the rounding of its sum, which the general window
+// deposits too where it isn't zero.
 template <int ORDER, class Reg>
 __device__ __forceinline__ void deposit_cross(const SmemAcc<Reg> &acc, const float o[3], const float d[3], const int s[3],
-                                              const float fac[3], int e)
+                                              const float fac[3], int e, const float v[3], const float h[3])
 {
     using S = Shape<ORDER>;
     constexpr int L = S::L, N = S::N;
     const int stride[3] = {1, acc.reg.rx(), acc.reg.r2()};
     const int a = e == 2 ? 0 : e + 1, b = a == 2 ? 0 : a + 1;
-    auto pickf = [](const auto *v, int i) { return i == 0 ? v[0] : (i == 1 ? v[1] : v[2]); };
+    auto pickf = [](const auto *p, int i) { return i == 0 ? p[0] : (i == 1 ? p[1] : p[2]); };
     const int se = pickf(stride, e), sa = pickf(stride, a), sb = pickf(stride, b);
     const float oe = pickf(o, e), de = pickf(d, e);
     const int she = pickf(s, e);
     float S0e[L], De[L], S0a[N], Da[N], S0b[N], Db[N];
     int ste, sta, stb;
-    S::general(oe, de, she, ste, S0e, De);
+    S::general(oe, de, she, pickf(v, e), pickf(h, e), ste, S0e, De);
     shapes_general<ORDER>(pickf(o, a), pickf(d, a), sta, S0a, Da);
     shapes_general<ORDER>(pickf(o, b), pickf(d, b), stb, S0b, Db);
-    float Ae[L], Qe[L], Fe[L - 1], Aa[N], Qa[N], Fa[N - 1], Ab[N], Qb[N], Fb[N - 1];
+    float Ae[L], Qe[L], Fe[L - 1], Aa[N], Qa[N], Fa[N], Ab[N], Qb[N], Fb[N];
     const float fe = pickf(fac, e) * acc.scale(e), fa = pickf(fac, a) * acc.scale(a), fb = pickf(fac, b) * acc.scale(b);
     float run = 0.f;
 #pragma unroll
@@ -74,7 +76,8 @@ __device__ __forceinline__ void deposit_cross(const SmemAcc<Reg> &acc, const flo
         Qb[i] = Db[i] * (1.f / 12.f);
         ra += Da[i];
         rb += Db[i];
-        if (i < N - 1) { Fa[i] = fa * ra; Fb[i] = fb * rb; }
+        Fa[i] = fa * ra;
+        Fb[i] = fb * rb;
     }
     const int at = acc.base + ste * se + sta * sa + stb * sb;
     const int pe = at + e * acc.reg.r3(), pa = at + a * acc.reg.r3(), pb = at + b * acc.reg.r3();
@@ -97,6 +100,8 @@ __device__ __forceinline__ void deposit_cross(const SmemAcc<Reg> &acc, const flo
                 acc.add(pa + k * sa + l * sb + m * se, Fa[k] * Ya);
                 acc.add(pb + k * sb + l * sa + m * se, Fb[k] * Yb);
             }
+            if (Fa[N - 1] != 0.f) acc.add(pa + (N - 1) * sa + l * sb + m * se, Fa[N - 1] * Ya);
+            if (Fb[N - 1] != 0.f) acc.add(pb + (N - 1) * sb + l * sa + m * se, Fb[N - 1] * Yb);
         }
 }
 
@@ -127,7 +132,12 @@ __device__ __forceinline__ void deposit_cross(const SmemAcc<Reg> &acc, const flo
 // ms per step, with the cell-ordered lanes -> one CTA of 512 threads -> two CTAs: plasma buncher
 // 5.22 -> 4.15 -> 3.80, sweep of 64 runs 18.0 -> 15.1 -> 13.6, long undulator 4.66 -> 4.19 -> 4.12, 65k
 // electrons CIC 0.045 -> 0.046 -> 0.033 (the region follows the drift), 2-D buncher 2.40 -> 1.40 (1.76 with one CTA: launch_push_dyn).
-template <int ORDER, int GATHER, int NT, int MINB, class Reg>
+// NEUTRAL: a species whose current another one's nearly cancels (see cancels).
+//  - Its crossings' last digit shows in the fields (see Shape), and a lattice that crosses takes its tiles'
+//    currents with it.  An item's first kQueue crossings are formed from the rounded displacement, the
+//    rest from the product it rounds, in the order of gq passes over the octants: 1.2e-3 of E lies between
+//    that and one form for all, for a lattice of 2 x 2 x 2 a cell of which half crosses.
+template <int ORDER, int GATHER, int NT, int MINB, bool NEUTRAL, class Reg>
 __global__ void __launch_bounds__(NT, MINB)
 k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work, int *work_sparse, int *err, Reg reg, int age)
 {
@@ -137,7 +147,8 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
     __shared__ int4 s_item;
     __shared__ float s_js[3], s_jinv[3], s_dl[3];
     __shared__ int s_lo[3], s_hi[3], s_sum[3], s_live, s_n;
-    __shared__ unsigned s_mark[kChunk / 32];      // listed records, a bit each
+    constexpr int PASSES = NEUTRAL ? 2 : 1;
+    __shared__ unsigned s_mark[PASSES][kChunk / 32];   // listed records, a bit each (in the order of the passes)
     const int Rx = reg.rx(), Ry = reg.ry(), R2 = reg.r2(), R3 = reg.r3(), Rz = R3 / R2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // dynamic shared memory: the currents' words and the fields; the list takes the fields' place when
@@ -162,7 +173,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             s_n = 0;
             s_live = 0;
         }
-        for (int l = tid; l < kChunk / 32; l += NT) s_mark[l] = 0u;
+        for (int l = tid; l < PASSES * (kChunk / 32); l += NT) s_mark[0][l] = 0u;
         if (tid < 3) {
             s_lo[tid] = 1 << 20;
             s_hi[tid] = -(1 << 20);
@@ -285,6 +296,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             return in;
         };
         const int len = p1 - p0;
+        const int gq = (len + kQueue - 1) / kQueue;
         const int K = max(1, min((item.w + 4 * t.tile_cells) / (8 * t.tile_cells), (len + 31) / 32));
         const int rounds = (len + 32 * K - 1) / (32 * K) * K;
         for (int rd = warp; rd < rounds; rd += NT / 32) {
@@ -296,22 +308,24 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             if (cell < 0) continue;
             int rel[3];
             if (!in_region(cell, rel)) {
-                atomicOr(&s_mark[q >> 5], 1u << (q & 31));
+                atomicOr(&s_mark[PASSES - 1][q >> 5], 1u << (q & 31));
                 continue;
             }
             float4 mo = sp.mom[p];
             const float o[3] = {R.x, R.y, R.z};
             int c[3] = {g.cc.i(cell), g.cc.j(cell), g.cc.k(cell)}, s[3];
             SmemAcc<Reg> acc{reg, sF, sJlo, sJhi, s_js, rel[2] * R2 + rel[1] * Rx + rel[0]};
-            float d[3], o1[3];
-            if (!push_move<ORDER, false, SmemAcc<Reg>, GATHER>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb)) {
+            float d[3], o1[3], v[3];
+            if (!push_move<ORDER, false, SmemAcc<Reg>, GATHER>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb, v)) {
                 sp.pos[p].w = __int_as_float(-1);
                 continue;
             }
             sp.mom[p] = mo;
             const bool fits = fabsf(d[0]) <= s_dl[0] && fabsf(d[1]) <= s_dl[1] && fabsf(d[2]) <= s_dl[2];
             if (!fits || !stays_all<ORDER>(o, d, s)) {
-                atomicOr(&s_mark[q >> 5], 1u << (q & 31));   // its position is still the old one
+                const int oct = (o[0] >= 0.5f) | ((o[1] >= 0.5f) << 1) | ((o[2] >= 0.5f) << 2);
+                const int pass = NEUTRAL ? 2 * (oct % gq) / gq : 0;
+                atomicOr(&s_mark[pass][q >> 5], 1u << (q & 31));   // its position is still the old one
                 continue;
             }
             sp.pos[p] = make_float4(o1[0], o1[1], o1[2], __int_as_float(g.cc.pack(c[0], c[1], c[2])));
@@ -322,15 +336,18 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
         }
         __syncthreads();
         // ---- listed records
-        for (int w = warp; w < (len + 31) / 32; w += NT / 32) {
-            const unsigned m = s_mark[w];
-            if (m == 0u) continue;
-            int at = 0;
-            if (lane == 0) at = atomicAdd(&s_n, __popc(m));
-            at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
-            if ((m >> lane) & 1u) list[at] = (unsigned short)(w * 32 + lane);
+#pragma unroll
+        for (int pass = 0; pass < PASSES; pass++) {
+            for (int w = warp; w < (len + 31) / 32; w += NT / 32) {
+                const unsigned m = s_mark[pass][w];
+                if (m == 0u) continue;
+                int at = 0;
+                if (lane == 0) at = atomicAdd(&s_n, __popc(m));
+                at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+                if ((m >> lane) & 1u) list[at] = (unsigned short)(w * 32 + lane);
+            }
+            __syncthreads();
         }
-        __syncthreads();
         const int n_list = s_n;
         for (int q = tid; q < n_list; q += NT) {
             const int p = p0 + list[q];
@@ -346,11 +363,14 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             int c[3] = {g.cc.i(cl), g.cc.j(cl), g.cc.k(cl)}, s[3];
             const int c0[3] = {c[0], c[1], c[2]};
             const float o[3] = {R.x, R.y, R.z};
-            float d[3], o1[3];
-            move(o, c, mo, g, err, d, s, o1, zb);   // it stays in the grid: the first loop's move has seen to that
+            float d[3], o1[3], v[3], h[3] = {g.dt_over_d[0], g.dt_over_d[1], g.dt_over_d[2]};
+            move(o, c, mo, g, err, d, s, o1, zb, v);   // it stays in the grid: the first loop's move has seen to that
             sp.pos[p] = make_float4(o1[0], o1[1], o1[2], __int_as_float(g.cc.pack(c[0], c[1], c[2])));
             const float fac[3] = {sp.cf[0] * mo.w, sp.cf[1] * mo.w, sp.cf[2] * mo.w};
             const bool fits = fabsf(d[0]) <= s_dl[0] && fabsf(d[1]) <= s_dl[1] && fabsf(d[2]) <= s_dl[2];
+            if (!NEUTRAL || q < kQueue)
+#pragma unroll
+                for (int k = 0; k < 3; k++) { v[k] = d[k]; h[k] = 1.f; }
             bool in = fits;
             int e = 0, crossed = 0;
 #pragma unroll
@@ -364,7 +384,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             }
             if (in && crossed == 1) {
                 const SmemAcc<Reg> acc{reg, sF, sJlo, sJhi, s_js, rel[2] * R2 + rel[1] * Rx + rel[0]};
-                deposit_cross<ORDER>(acc, o, d, s, fac, e);
+                deposit_cross<ORDER>(acc, o, d, s, fac, e, v, h);
                 continue;
             }
             // several dims (its window's tests need every dim), beyond the range or the region
@@ -375,7 +395,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             }
             if (in) {
                 SmemAcc<Reg> acc{reg, sF, sJlo, sJhi, s_js, rel[2] * R2 + rel[1] * Rx + rel[0]};
-                deposit_general<ORDER>(acc, o, d, s, fac);
+                deposit_general<ORDER>(acc, o, d, s, fac, v, h);
             } else {
                 GlobAcc<ORDER> acc(f, g, c0, err, zb);
                 deposit_general<ORDER>(acc, o, d, s, fac);
@@ -442,13 +462,13 @@ inline size_t push_smem(int R3) { return (size_t)24 * R3 + std::max((size_t)24 *
 // Steps since the species' last sort.
 inline int sort_age(const pic_ctx *c) { return (int)((c->step - c->sort_base) % c->sort_every); }
 
-template <int ORDER, int GATHER, int NT, int MINB, class Reg>
+template <int ORDER, int GATHER, int NT, int MINB, bool NEUTRAL = false, class Reg>
 cudaError_t launch_push_t(pic_ctx *c, int si, const ExtDev &ext, Reg reg, int R3)
 {
     static KernelCache cache;
     const Species &s = c->sp[si];
     const size_t smem = push_smem(R3);
-    auto kern = k_push<ORDER, GATHER, NT, MINB, Reg>;
+    auto kern = k_push<ORDER, GATHER, NT, MINB, NEUTRAL, Reg>;
     int per_sm = 0;
     cudaError_t e = cache.blocks_per_sm((const void *)kern, c->dev.device, NT, smem, &per_sm);
     if (e != cudaSuccess) return e;
@@ -466,6 +486,7 @@ template <int ORDER, int GATHER> cudaError_t launch_push_fixed(pic_ctx *c, int s
     // cost.  Small ones, an item or two per CTA, end with their longest thread: 2 x 256 at 128 (300k
     // electrons 0.100 against 0.112 ms per step, 500k 0.115 / 0.130, 3.4M plasma 0.350 / 0.343).
     const RegFix<R, R, R, R2> reg;
+    if (cancels(c, si)) return launch_push_t<ORDER, GATHER, 512, 2, true>(c, si, ext, reg, R2 * R);
     if (c->sp[si].bound <= 8192 * (int64_t)c->num_sms) return launch_push_t<ORDER, GATHER, 256, 2>(c, si, ext, reg, R2 * R);
     return launch_push_t<ORDER, GATHER, 512, 2>(c, si, ext, reg, R2 * R);
 }
@@ -482,7 +503,7 @@ template <int ORDER, int GATHER> cudaError_t launch_push_dyn(pic_ctx *c, int si,
     // order in which neighbouring tiles flush, and the smaller the tiles the more of its nodes are
     // shared.  One CTA an SM keeps neighbours in the items' order (2-D buncher, 8 x 1 x 8 tiles: 1.76 ms
     // per step against 1.18 with four CTAs, with a fourth of the scatter of B between launches).
-    if (c->plasma && si == c->sp_e) return launch_push_t<ORDER, GATHER, 512, 1>(c, si, ext, reg, R3);
+    if (cancels(c, si)) return launch_push_t<ORDER, GATHER, 512, 1, true>(c, si, ext, reg, R3);
     if (4 * cta <= sm) return launch_push_t<ORDER, GATHER, 128, 4>(c, si, ext, reg, R3);
     if (2 * cta <= sm) return launch_push_t<ORDER, GATHER, 256, 2>(c, si, ext, reg, R3);
     return launch_push_t<ORDER, GATHER, 512, 1>(c, si, ext, reg, R3);

@@ -1,0 +1,140 @@
+"""Currents of particles that change their nearest node, to the last bit.
+
+A cold lattice crosses all at once and rounds alike, and a neutral plasma's electrons and ions nearly
+cancel, so the last digit of a crossing particle's current shows in the fields.  The reference here is
+the deposit restated operation by operation in numpy's FP32 (the general Esirkepov window, the item's
+fixed point, its flush); no tolerance.
+"""
+import numpy as np
+import pytest
+
+from paper_2411_04703_gb300 import api
+
+pytestmark = pytest.mark.gpu
+
+F = np.float32
+GRID, TILE, DT = 48, 8, F(0.4375)
+QUEUE, CHUNK, CHUNK_MIN = 1024, 4096, 512     # first crossings of an item, records of an item
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+
+
+def _fma(a, b, c):
+    # the product of two FP32 values is exact in FP64
+    return (a.astype(np.float64) * b + c).astype(F)
+
+
+def _shape(order, t):
+    a = np.abs(t)
+    if order == 1:
+        return np.maximum(F(0), F(1) - a)
+    return np.where(a <= F(0.5), _fma(-a, a, F(0.75)), F(0.5) * (F(1.5) - a) * (F(1.5) - a) * (a < F(1.5)))
+
+
+def _slope(order, t):
+    a = np.abs(t)
+    if order == 1:
+        return np.where(a < 1, np.where(t > 0, F(-1), np.where(t < 0, F(1), F(0))), F(0))
+    s = np.where(a <= F(0.5), F(-2) * a, np.where(a < F(1.5), a - F(1.5), F(0)))
+    return np.where(t < 0, -s, s)
+
+
+def _general(order, o, d, v, h):
+    """First node and the values S0, DS on the general window's order + 2 nodes of one dim."""
+    half = F(0) if order == 1 else F(0.5)
+    b0, b1 = np.floor(o + half), np.floor(o + d + half)
+    st = np.minimum(b0, b1) - (order - 1)
+    S0, DS = [], []
+    for a in range(order + 2):
+        t0 = o - (st + a).astype(F)
+        t1 = t0 + d
+        lo, hi = np.minimum(t0, t1), np.maximum(t0, t1)
+        k = np.ceil(hi - half) - F(1) + half
+        p = ((st + a).astype(F) + k) - o
+        b = _fma(v, h, -p)
+        two = _fma(p, _slope(order, k - F(0.5) * p), (b * _slope(order, k + F(0.5) * b)).astype(np.float64))
+        S0.append(_shape(order, t0))
+        DS.append(np.where(k > lo, two, d * _slope(order, t0 + F(0.5) * d)))
+    return st.astype(int), np.array(S0), np.array(DS)
+
+
+def _fixed(order, o, d, v, h, fs):
+    """Fixed-point contributions of one particle: window's first node [3, n], values [3][x][y][z][n]."""
+    L = order + 2
+    w = [_general(order, o[k], d[k], v[k], h) for k in range(3)]
+    A = [_fma(F(0.5) * np.ones_like(w[k][2]), w[k][2], w[k][1]) for k in range(3)]
+    Q = [w[k][2] * F(1.0 / 12.0) for k in range(3)]
+    P = []
+    for k in range(3):
+        run, rows = np.zeros_like(o[0]), []
+        for a in range(L):
+            run = run + w[k][2][a]
+            rows.append(fs[k] * run if a < L - 1 else np.zeros_like(run))
+        P.append(np.array(rows))
+    out = []
+    for k in range(3):
+        a, b = (k + 1) % 3, (k + 2) % 3
+        Y = _fma(A[a][:, None], A[b][None], (Q[a][:, None] * w[b][2][None]).astype(np.float64))
+        V = np.rint(P[k][:, None, None] * Y[None]).astype(np.int64)          # [k, a, b, n]
+        out.append(np.moveaxis(V, [0, 1, 2], [k, a, b]))
+    return np.stack([w[k][0] for k in range(3)]), np.array(out)
+
+
+@pytest.mark.parametrize("order", [1, 2])
+@pytest.mark.parametrize("copies", [40, CHUNK])
+@pytest.mark.parametrize("neutral", [False, True])
+def test_crossing_currents_bit_by_bit(order, copies, neutral):
+    # every tile holds copies of one particle; of a neutral species' item the first QUEUE crossings take
+    # the length behind a knot from the rounded displacement, the others from the product it rounds
+    import torch
+    rng = np.random.default_rng(100 * order + copies)
+    nt = GRID // TILE
+    cell = np.stack(np.meshgrid(*[np.arange(nt)] * 3, indexing="ij")).reshape(3, -1) * TILE + 4
+    n = cell.shape[1]
+    o = rng.random((3, n)).astype(F)
+    u = (rng.integers(-32, 33, (3, n)) / 8.0).astype(F)                       # 1 + u^2 is exact in FP32
+    x = np.repeat(cell + o.astype(np.float64), copies, axis=1)
+    wt = F(2.0 ** -10)
+    sim = api.Sim((GRID,) * 3, (1.0,) * 3, float(DT), 2.0, order=order)
+    sim.load_species(-1.0, 1.0, x, np.repeat(u.astype(np.float64), copies, axis=1), np.full(n * copies, float(wt)),
+                     frame=api.PIC_FRAME_BOOSTED)
+    if neutral:
+        sim.load_species(1.0, 1836.0)                                         # none of them yet
+    sim.step(1)
+    sim.sync()
+    J = np.stack([sim.get_field(api.PIC_JX + k) for k in range(3)])           # [c, z, y, x]
+
+    ig = torch.rsqrt(torch.tensor(1.0 + (u.astype(np.float64) ** 2).sum(0), dtype=torch.float32, device="cuda")).cpu().numpy()
+    v = u * ig
+    d = v * DT
+    near = F(0) if order == 1 else F(0.5)
+    crosses = (np.floor(o + d + near) != np.floor(o + near)).any(0)
+    assert 40 < crosses.sum() < n
+    cf = F(1.0 / float(DT))
+    fac = cf * wt
+    dlim = min(DT, F(4) * np.abs(d).max())
+    js = F(2.0 ** (30 - np.frexp(F(1.1) * cf * wt * dlim)[1]))
+    fs = [fac * js] * 3
+    st, near_form = _fixed(order, o, d, d, F(1), fs)
+    _, far_form = _fixed(order, o, d, v, DT, fs)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count * (1 if neutral else 2)
+    chunk = CHUNK
+    while chunk > CHUNK_MIN and n * copies // chunk < sms:
+        chunk //= 2
+    want = np.zeros_like(near_form, dtype=F)
+    for first in range(0, copies, chunk):
+        length = min(chunk, copies - first)
+        a = min(length, QUEUE) if neutral else length
+        total_hi = a * (near_form >> 19) + (length - a) * (far_form >> 19)
+        total_lo = a * (near_form & 0x7FFFF) + (length - a) * (far_form & 0x7FFFF)
+        want = want + ((total_hi.astype(np.float64) * 2.0 ** 19 + total_lo.astype(F)).astype(F) * (F(1) / js))
+    for q in np.flatnonzero(crosses):
+        x0, y0, z0 = (cell[:, q] + st[:, q])
+        got = J[:, z0:z0 + order + 2, y0:y0 + order + 2, x0:x0 + order + 2]
+        ref = np.swapaxes(want[..., q], 1, 3)
+        assert np.array_equal(got, ref), (q, o[:, q], d[:, q], np.abs(got - ref).max() / np.abs(ref).max())
