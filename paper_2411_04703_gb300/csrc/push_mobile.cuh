@@ -137,7 +137,12 @@ __device__ __forceinline__ void deposit_cross(const SmemAcc<Reg> &acc, const flo
 //    currents with it.  An item's first kQueue crossings are formed from the rounded displacement, the
 //    rest from the product it rounds, in the order of gq passes over the octants: 1.2e-3 of E lies between
 //    that and one form for all, for a lattice of 2 x 2 x 2 a cell of which half crosses.
-template <int ORDER, int GATHER, int NT, int MINB, bool NEUTRAL, class Reg>
+// INORDER: its tiles' currents are added to the other's, each addition rounded at that one's size, so a
+// shared node depends on which of its tiles flushes first.  With one CTA an SM, and an item claimed when
+// the one before it is flushed, neighbours flush in the order of the items.  An item claimed ahead lets
+// the CTAs drift apart, and two CTAs flush twice as many tiles at once: two launches of one state then
+// differ 2 to 4 times as much (J of 76 x 78 x 298 cells at 4 a cell, 4 steps: 1.4e-5, 6.4e-5 so).
+template <int ORDER, int GATHER, int NT, int MINB, bool NEUTRAL, bool INORDER, class Reg>
 __global__ void __launch_bounds__(NT, MINB)
 k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work, int *work_sparse, int *err, Reg reg, int age)
 {
@@ -162,14 +167,16 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
     const long long gnx = g.n[0], gnxy = (long long)g.n[0] * g.n[1];
     unsigned dmax[3] = {0u, 0u, 0u};
 
-    if (tid == 0) {
+    auto claim = [&]() {
         const int it = atomicAdd(work, 1);
         s_item = it < n_items ? t.items[it] : make_int4(-1, 0, 0, 0);
-    }
+    };
+    if (!INORDER && tid == 0) claim();
     for (int l = tid; l < 6 * R3; l += NT) sJlo[l] = 0u;   // both words; a flush leaves them zero again
     for (;;) {
         if (tid == 0) {
-            cp_async_wait();                       // s_item
+            if (INORDER) claim();
+            else cp_async_wait();                  // s_item
             s_n = 0;
             s_live = 0;
         }
@@ -183,7 +190,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
         const int4 item = s_item;
         if (item.x < 0) break;
         int it = 0;
-        if (tid == 0) it = atomicAdd(work, 1);     // the next item's number, and behind the staging its record
+        if (!INORDER && tid == 0) it = atomicAdd(work, 1);   // the next item's number, and behind the staging its record
         const int tile = item.x, p0 = item.y, p1 = item.z;
         const int t0[3] = {(tile % t.nt[0]) * t.T[0], ((tile / t.nt[0]) % t.nt[1]) * t.T[1], (tile / (t.nt[0] * t.nt[1])) * t.T[2]};
         const int zb = g.nzr == g.n[2] ? 0 : zblock(t0[2], g.nzr);
@@ -278,7 +285,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
         }
         cp_async_wait();
         __syncthreads();
-        if (tid == 0) {
+        if (!INORDER && tid == 0) {
             if (it < n_items) cp_async16(&s_item, t.items + it);
             else s_item.x = -1;
         }
@@ -462,13 +469,13 @@ inline size_t push_smem(int R3) { return (size_t)24 * R3 + std::max((size_t)24 *
 // Steps since the species' last sort.
 inline int sort_age(const pic_ctx *c) { return (int)((c->step - c->sort_base) % c->sort_every); }
 
-template <int ORDER, int GATHER, int NT, int MINB, bool NEUTRAL = false, class Reg>
+template <int ORDER, int GATHER, int NT, int MINB, bool NEUTRAL = false, bool INORDER = false, class Reg>
 cudaError_t launch_push_t(pic_ctx *c, int si, const ExtDev &ext, Reg reg, int R3)
 {
     static KernelCache cache;
     const Species &s = c->sp[si];
     const size_t smem = push_smem(R3);
-    auto kern = k_push<ORDER, GATHER, NT, MINB, NEUTRAL, Reg>;
+    auto kern = k_push<ORDER, GATHER, NT, MINB, NEUTRAL, INORDER, Reg>;
     int per_sm = 0;
     cudaError_t e = cache.blocks_per_sm((const void *)kern, c->dev.device, NT, smem, &per_sm);
     if (e != cudaSuccess) return e;
@@ -486,7 +493,7 @@ template <int ORDER, int GATHER> cudaError_t launch_push_fixed(pic_ctx *c, int s
     // cost.  Small ones, an item or two per CTA, end with their longest thread: 2 x 256 at 128 (300k
     // electrons 0.100 against 0.112 ms per step, 500k 0.115 / 0.130, 3.4M plasma 0.350 / 0.343).
     const RegFix<R, R, R, R2> reg;
-    if (cancels(c, si)) return launch_push_t<ORDER, GATHER, 512, 2, true>(c, si, ext, reg, R2 * R);
+    if (cancels(c, si)) return launch_push_t<ORDER, GATHER, 512, 1, true, true>(c, si, ext, reg, R2 * R);
     if (c->sp[si].bound <= 8192 * (int64_t)c->num_sms) return launch_push_t<ORDER, GATHER, 256, 2>(c, si, ext, reg, R2 * R);
     return launch_push_t<ORDER, GATHER, 512, 2>(c, si, ext, reg, R2 * R);
 }
@@ -503,6 +510,7 @@ template <int ORDER, int GATHER> cudaError_t launch_push_dyn(pic_ctx *c, int si,
     // order in which neighbouring tiles flush, and the smaller the tiles the more of its nodes are
     // shared.  One CTA an SM keeps neighbours in the items' order (2-D buncher, 8 x 1 x 8 tiles: 1.76 ms
     // per step against 1.18 with four CTAs, with a fourth of the scatter of B between launches).
+    if (cancels(c, si) && c->n[1] > 1) return launch_push_t<ORDER, GATHER, 512, 1, true, true>(c, si, ext, reg, R3);
     if (cancels(c, si)) return launch_push_t<ORDER, GATHER, 512, 1, true>(c, si, ext, reg, R3);
     if (4 * cta <= sm) return launch_push_t<ORDER, GATHER, 128, 4>(c, si, ext, reg, R3);
     if (2 * cta <= sm) return launch_push_t<ORDER, GATHER, 256, 2>(c, si, ext, reg, R3);

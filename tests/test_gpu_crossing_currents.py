@@ -138,3 +138,19 @@ def test_crossing_currents_bit_by_bit(order, copies, neutral):
         got = J[:, z0:z0 + order + 2, y0:y0 + order + 2, x0:x0 + order + 2]
         ref = np.swapaxes(want[..., q], 1, 3)
         assert np.array_equal(got, ref), (q, o[:, q], d[:, q], np.abs(got - ref).max() / np.abs(ref).max())
+
+
+def test_neutral_plasma_spread_of_two_runs():
+    # the plasma's tiles add to the ions' current, which theirs nearly cancels, and each addition rounds at
+    # its size: two runs of one state differ by the order in which neighbouring tiles are added.  Bound:
+    # twice the 1.4e-5 that J of this run differs by where tiles are added in the order of the work items.
+    from paper_2411_04703_gb300 import workloads as W
+    runs = []
+    for _ in range(2):
+        w = W.plasma_buncher(grid=(76, 78, 298), n_beam=59539, seed=7, pml=10, ppc=(1, 2, 2))
+        sim, _ids = api.from_workload(w)
+        sim.step(4)
+        sim.sync()
+        runs.append(np.stack([sim.get_field(api.PIC_JX + k) for k in range(3)]).astype(np.float64))
+        sim.close()
+    assert np.linalg.norm(runs[1] - runs[0]) < 2 * 1.4e-5 * np.linalg.norm(runs[0])
