@@ -288,7 +288,7 @@ struct MomP {
     double shifts, tp, gR, bR, igR2, mass, k;
     int frame;
     double mean_t;
-    double about[7];  // x y z ux uy uz gamma of the mean particle
+    double about[7];  // x y z ux uy uz gamma: the means of pass 0 in the frame
     CellCode cc;
     int k_lo, k_hi;   // rows of the run whose particles are summed (ensembles; whole grid otherwise)
 };
@@ -325,10 +325,12 @@ __device__ __forceinline__ void particle_frame(const MomP &p, float4 P, float4 M
 }
 
 // Two passes.  FP64 arithmetic bounds them (2 operations per clock and SM: a particle's frame costs
-// ~150, the phase's sincos as many): pass 0 is kept to the weights, the time and the stored means, and
-// pass 1 takes first and second moments at once, about the mean particle's own transform.  That is so near
-// the mean that the shift back costs no digit.  Both frames' moments of 2M particles and a charge density:
-// 3,799 us with three passes that each worked out the frame, 3,418 us with these.
+// ~150, the phase's sincos as many): pass 0 is kept to the weights, the time and the means of the stored
+// position, momentum and their Lorentz factor, and pass 1 takes first and second moments at once, about
+// the transform of those means.  It is linear in them, so that momenta and Lorentz factor are taken about
+// their means to rounding, and the shift back costs no digit; a lab position is about the mean before its
+// drift to the mean time, which is within the spread.  (About the Lorentz factor of the mean momentum
+// instead, 0.5 from the mean for a beam in an undulator of K = 1, an energy spread of 1e-5 loses 4 digits.)
 template <int PASS> __global__ void k_moments(SpeciesDev sp, MomP p, double *partial)
 {
     double acc[kMomK];
@@ -351,6 +353,8 @@ template <int PASS> __global__ void k_moments(SpeciesDev sp, MomP p, double *par
             acc[2] += 1.0;
             acc[3] += w * x; acc[4] += w * y; acc[5] += w * z;
             acc[6] += w * Mo.x; acc[7] += w * Mo.y; acc[8] += w * Mo.z;
+            const double ux = Mo.x, uy = Mo.y, uz = Mo.z;
+            acc[9] += w * sqrt(1.0 + ux * ux + uy * uy + uz * uz);
         } else {
             double x[3], u[3], g, t;
             particle_frame(p, P, Mo, x, u, g, t);
@@ -661,10 +665,9 @@ cudaError_t launch_moments(pic_ctx *c, const Species &s, int frame, double k, do
             const double sw = sums[0][0];
             p.mean_t = sw > 0 ? sums[0][1] / sw : p.tp;
             if (sw > 0) {
-                // the mean particle in the frame (its time is the mean time)
+                // the means in the frame (the time is the mean time)
                 const double *m = sums[0] + 3;
-                const double zp = m[2] / sw, ux = m[3] / sw, uy = m[4] / sw, uz = m[5] / sw;
-                const double gp = sqrt(1.0 + ux * ux + uy * uy + uz * uz);
+                const double zp = m[2] / sw, ux = m[3] / sw, uy = m[4] / sw, uz = m[5] / sw, gp = m[6] / sw;
                 const bool lab = frame == PIC_FRAME_LAB;
                 const double about[7] = {m[0] / sw, m[1] / sw, lab ? p.gR * (zp + p.bR * p.tp) : zp, ux, uy,
                                          lab ? p.gR * (uz + p.bR * gp) : uz, lab ? p.gR * (gp + p.bR * uz) : gp};

@@ -95,3 +95,26 @@ def test_moments_in_two_passes(n, umax, frame, oframe):
         assert g[k] == pytest.approx(r[k], rel=1e-9, abs=1e-12), (k, g[k], r[k])
     for k in ("rms_x", "rms_y", "rms_z", "rel_energy_spread", "emit_nx", "emit_ny"):
         assert g[k] == pytest.approx(r[k], rel=1e-9, abs=1e-7 * scale), (k, g[k], r[k])
+
+
+# A small energy spread beside a large transverse momentum: the Lorentz factor of the mean momentum is far
+# from the mean one.  Bound: a record's Lorentz factor in its frame is some eight FP64 roundings, and the
+# spread about their mean no further off than they are, 8 x 1.1e-16 of the mean, times ten.
+@pytest.mark.parametrize("frame", [api.PIC_FRAME_LAB, api.PIC_FRAME_BOOSTED])
+@pytest.mark.parametrize("ux, uz", [(1.0, 3.0), (100.0, 0.5), (0.5, -20.0)])
+def test_energy_spread_beside_a_transverse_oscillation(frame, ux, uz):
+    w = W.vacuum_undulator(grid=(20, 10, 18), n_beam=4, seed=3, order=2)
+    sim, _ = api.from_workload(w, beam=False)
+    n, rng = 20000, np.random.default_rng(5)
+    X = rng.uniform(4.0, 9.0, (3, n)) * np.array(w.d)[:, None]
+    U = np.stack([ux * np.where(np.arange(n) % 2, 1.0, -1.0), np.zeros(n), uz * (1.0 + 1e-6 * rng.standard_normal(n))])
+    sid = sim.load_species(-1.0, 1.0, X, U, np.ones(n), frame=api.PIC_FRAME_BOOSTED)
+    u = sim.get_particles(sid)["u"].astype(np.longdouble)
+    g = np.sqrt(1 + (u ** 2).sum(1))
+    if frame == api.PIC_FRAME_LAB:
+        gR = np.longdouble(w.gamma_R)
+        g = gR * (g + np.sqrt(1 - 1 / gR ** 2) * u[:, 2])
+    spread = float(np.sqrt(((g - g.mean()) ** 2).mean()) / g.mean())
+    m = sim.get_moments(sid, frame, k_bunch=3.0)
+    assert m["mean_gamma"] == pytest.approx(float(g.mean()), rel=1e-13)
+    assert abs(m["rel_energy_spread"] - spread) < 80 * 1.1e-16, (m["rel_energy_spread"], spread)
