@@ -36,10 +36,12 @@ __global__ void k_lattice_step(LatStepP p, int *err)
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < p.cap; s += (long long)gridDim.x * blockDim.x) {
         PlaneRec r = p.planes[s];
         if (r.kz < 0) continue;
-        // the move of a frozen particle with u = (0, 0, u_z), in the particle kernel's FP32 steps
+        // the move of a frozen particle with u = (0, 0, u_z); the roundings are spelt out, because a
+        // plasma's current is what is left of this one and the electrons' (the sum rounds twice, where
+        // the particle kernel's move rounds once)
         const float ig = rsqrtf(1.f + p.uz * p.uz);
-        const float d = p.uz * ig * p.dtdz;
-        const float x1 = r.oz + d;
+        const float d = __fmul_rn(__fmul_rn(p.uz, ig), p.dtdz);
+        const float x1 = __fadd_rn(r.oz, d);
         int sh = (int)floorf(x1);
         float o1 = x1 - (float)sh;
         if (o1 >= 1.f) { o1 = 0.f; sh += 1; }

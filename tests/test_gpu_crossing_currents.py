@@ -154,3 +154,21 @@ def test_neutral_plasma_spread_of_two_runs():
         runs.append(np.stack([sim.get_field(api.PIC_JX + k) for k in range(3)]).astype(np.float64))
         sim.close()
     assert np.linalg.norm(runs[1] - runs[0]) < 2 * 1.4e-5 * np.linalg.norm(runs[0])
+
+
+def test_lattice_ions_move_bit_by_bit():
+    # their offsets are pinned like the electrons' currents: the sum of offset and displacement, rounded
+    import torch
+    grid, dt, gR = (12, 12, 24), F(0.40625), 1.25                             # u_z = -0.75: 1 + u_z^2 is exact
+    sim = api.Sim(grid, (1.0, 1.0, 1.0), float(dt), gR, order=2)
+    _, ions = sim.set_plasma((1, 1, 3), (0, 12, 0, 12), (0.0, 1e3), (1e-3, 1e-3))
+    P = sim.get_particles(ions)
+    z = P["off"][np.argsort(P["id"]), 2]
+    ig = torch.rsqrt(torch.tensor(1.5625, dtype=torch.float32, device="cuda")).item()
+    d = F(-0.75) * F(ig) * dt
+    for _ in range(7):
+        sim.step(1)
+        z = z + d
+        z = z - np.floor(z)
+    P = sim.get_particles(ions)
+    assert np.array_equal(P["off"][np.argsort(P["id"]), 2], np.where(z >= 1, F(0), z))
