@@ -514,14 +514,15 @@ __device__ __forceinline__ bool move(const float o[3], int c[3], const float4 &m
                                      int s[3], float o1[3], int zb, float v[3])
 {
     const float u[3] = {mo.x, mo.y, mo.z};
-    const float ig = rsqrtf(1.f + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    const float ig = rsqrtf(fmaf(u[2], u[2], fmaf(u[1], u[1], fmaf(u[0], u[0], 1.f))));
     if (!(ig > 0.f)) { atomicOr(err, ERR_NAN); return false; }
     bool alive = true;
 #pragma unroll
     for (int dd = 0; dd < 3; dd++) {
         // the displacement of the push (cells), and the new offset with one rounding; both are spelt
-        // out, so that every path (and build) moves a particle to the same place: a cold lattice's
-        // particles round alike, and a neutral plasma's current is a small difference of large ones
+        // out, so that every path (and build) of the particle kernels moves a particle to the same
+        // place: a cold lattice's particles round alike, and a neutral plasma's current is a small
+        // difference of large ones
         v[dd] = __fmul_rn(u[dd], ig);
         d[dd] = __fmul_rn(v[dd], g.dt_over_d[dd]);
         const float x1 = fmaf(v[dd], g.dt_over_d[dd], o[dd]);

@@ -371,7 +371,10 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             const int c0[3] = {c[0], c[1], c[2]};
             const float o[3] = {R.x, R.y, R.z};
             float d[3], o1[3], v[3], h[3] = {g.dt_over_d[0], g.dt_over_d[1], g.dt_over_d[2]};
-            move(o, c, mo, g, err, d, s, o1, zb, v);   // it stays in the grid: the first loop's move has seen to that
+            if (!move(o, c, mo, g, err, d, s, o1, zb, v)) {   // (as in the first loop, which lists none that leaves)
+                sp.pos[p].w = __int_as_float(-1);
+                continue;
+            }
             sp.pos[p] = make_float4(o1[0], o1[1], o1[2], __int_as_float(g.cc.pack(c[0], c[1], c[2])));
             const float fac[3] = {sp.cf[0] * mo.w, sp.cf[1] * mo.w, sp.cf[2] * mo.w};
             const bool fits = fabsf(d[0]) <= s_dl[0] && fabsf(d[1]) <= s_dl[1] && fabsf(d[2]) <= s_dl[2];
