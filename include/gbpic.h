@@ -301,7 +301,9 @@ int pic_sync(pic_ctx *ctx);
 
 /* Force a per-tile sort of every species now (the sort also compacts dummy particles).  Order:
  * tiles x-fastest; inside a tile the cells x fastest, then z, then y; inside a cell the octant
- * of the offset (bit d set when offset_d >= 1/2); order among equal keys unspecified. */
+ * of the offset (bit d set when offset_d >= 1/2); order among equal keys unspecified.  The sorts
+ * inside pic_step put the octant of a mobile species before z and x, which its kernel reads faster:
+ * the steps from here to the next such sort take up to 14 % longer. */
 int pic_sort(pic_ctx *ctx);
 
 /* Copy one grid component (PIC_EX..PIC_JZ; J is the current of the last step) or the charge

@@ -390,7 +390,6 @@ TileDev tile_dev(const pic_ctx *c, const Species &s)
     t.M = c->M;
     t.hl = margin_lo(c);
     for (int d = 0; d < 3; d++) t.R[d] = c->T[d] + 2 * c->M + margin_lo(c) + margin_hi(c);
-    t.cell_start = s.cell_start;
     t.tile_start = s.tile_start;
     t.items = s.items;
     t.sparse_tiles = s.sparse_tiles;

@@ -15,8 +15,7 @@ namespace gbpic {
 constexpr int kMaxSpecies = 8;
 constexpr int kChunk = 4096;         // particles per work item of the particle kernel (at most)
 constexpr int kChunkMin = 512;       // smallest work item (small species are split finer)
-constexpr int kPushThreads = 1024;   // 32 warps per SM at 64 registers (measured 3 % faster than 512 at 122)
-constexpr int kGroup = kChunk / kPushThreads;   // consecutive particles of one lane per work item
+constexpr int kPushThreads = 1024;   // threads of the frozen species' kernel
 constexpr int kSparse = 32;   // a tile with fewer particles takes the global-memory path, one warp per tile
 
 // Error bits of the device error word.
@@ -133,8 +132,6 @@ struct TileDev {
     int M;                // allowed drift outside the tile between sorts (cells)
     int hl;               // stencil reach below the particle cell (1 CIC, 2 TSC)
     int R[3];             // shared-memory region size per dim
-    const int *cell_start;   // [n_keys + 1]: first sorted slot of each key (8 keys per cell), valid
-                             // for the tiles holding particles at the last sort
     const int *tile_start;   // [ntiles + 1]: first sorted slot of each tile (the last: the live count)
     const int4 *items;       // work items of the tiles with >= kSparse particles: tile, first slot, end slot, particles of the tile
     const int *sparse_tiles; // tiles with 1 .. kSparse-1 particles (count[3] of them)

@@ -4,7 +4,7 @@
 
 namespace gbpic {
 
-cudaError_t launch_push1_frozen(pic_ctx *c, int si, const ExtDev &ext) { return push::launch_frozen<1>(c, si, ext); }
+cudaError_t launch_push1_frozen(pic_ctx *c, int si) { return push::launch_frozen<1>(c, si); }
 cudaError_t launch_push1_fixed(pic_ctx *c, int si, const ExtDev &ext) { return push::launch_push_fixed<1, 0>(c, si, ext); }
 cudaError_t launch_push1_fixed_ec(pic_ctx *c, int si, const ExtDev &ext) { return push::launch_push_fixed<1, 1>(c, si, ext); }
 

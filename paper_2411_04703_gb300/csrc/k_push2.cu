@@ -4,12 +4,12 @@
 
 namespace gbpic {
 
-cudaError_t launch_push1_frozen(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push1_frozen(pic_ctx *c, int si);
 cudaError_t launch_push1_fixed(pic_ctx *c, int si, const ExtDev &ext);
 cudaError_t launch_push1_fixed_ec(pic_ctx *c, int si, const ExtDev &ext);
 cudaError_t launch_push1_dyn(pic_ctx *c, int si, const ExtDev &ext);
 cudaError_t launch_push1_dyn_ec(pic_ctx *c, int si, const ExtDev &ext);
-cudaError_t launch_push2_frozen(pic_ctx *c, int si, const ExtDev &ext);
+cudaError_t launch_push2_frozen(pic_ctx *c, int si);
 cudaError_t launch_push2_fixed(pic_ctx *c, int si, const ExtDev &ext);
 cudaError_t launch_push2_fixed_ec(pic_ctx *c, int si, const ExtDev &ext);
 cudaError_t launch_push2_dyn(pic_ctx *c, int si, const ExtDev &ext);
@@ -138,7 +138,7 @@ cudaError_t launch_dlim_from_momenta(pic_ctx *c, int si)
 cudaError_t launch_push(pic_ctx *c, int si, const ExtDev &ext)
 {
     const bool o1 = c->order == 1;
-    if (c->sp[si].frozen) return o1 ? launch_push1_frozen(c, si, ext) : launch_push2_frozen(c, si, ext);
+    if (c->sp[si].frozen) return o1 ? launch_push1_frozen(c, si) : launch_push2_frozen(c, si);
     const bool ec = c->gather == PIC_GATHER_ENERGY;
     if (push::default_region(c)) {
         if (o1) return ec ? launch_push1_fixed_ec(c, si, ext) : launch_push1_fixed(c, si, ext);

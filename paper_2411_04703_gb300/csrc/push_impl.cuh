@@ -1,5 +1,5 @@
-// Fused particle kernel of one boosted-frame PIC step (sm_103a): implementation shared by the
-// CIC (k_push1.cu) and TSC (k_push2.cu) translation units.
+// Particle kernels of one boosted-frame PIC step (sm_103a): the parts that the mobile species' kernel
+// (push_mobile.cuh) and the frozen species' kernel (below) share, and the latter.
 //
 // Per particle: gather E^n, B^n with the particle shape at each component's Yee point, add
 // the analytic external undulator field of the RRF (Eq. M1-M4 applied to the lab field at
@@ -7,18 +7,19 @@
 // move x^n -> x^{n+1} (integer cell + FP32 offset), and the Esirkepov charge-conserving current
 // J^{n+1/2} (Eq. Max3-Max4 solved by current weighting).
 //
-// Work decomposition: particles are sorted by tile; a persistent grid pulls (tile, chunk)
-// work items from an atomic counter.  For a tile item the CTA stages the E/B region of the
-// tile (+ drift margin + stencil halo) in shared memory, accumulates the current of its
-// particles in a shared-memory J region with shared atomics, and flushes the region to the
-// global J once with global atomics.  Particles that drifted beyond the margin since the last
-// sort, and appended (unsorted) particles, take the global-memory path.
+// Work decomposition: particles are sorted by tile; a persistent grid pulls work items (a chunk of a
+// tile's particles) from an atomic counter.  The CTA accumulates its particles' current in a region of
+// the tile (+ drift margin + stencil halo) in shared memory with shared atomics, and flushes it to the
+// global J once with global atomics; for mobile species it stages the region's E and B there first.
+// Particles outside the region, in tiles of a few, and appended since the sort take the global-memory
+// path.
 //
 // Deposit split: a particle whose nearest node (TSC) or cell (CIC) does not change in any
 // dimension during the step -- all but a few percent in a cold drifting plasma -- has its
 // Esirkepov current on a window of order+1 nodes per dimension with DS in closed form
-// (54 node updates for TSC instead of 144); the others are queued in shared memory and
-// deposited with the general window of order+2 nodes after the main loop.
+// (54 node updates for TSC instead of 144); the others are taken after the main loop, of mobile
+// species those that cross along one dim on a window a node longer along it, the rest on the general
+// window of order+2 nodes.
 #pragma once
 
 #include <mutex>
@@ -608,8 +609,6 @@ __device__ __forceinline__ void step_global(const SpeciesDev &sp, const GridDev 
 
 // Linear index of grid node (x, y, z) with periodic wrap (z inside the run starting at row zb),
 // or -1 outside a non-periodic face.
-__device__ __forceinline__ long long wrap_node(const GridDev &g, int x, int y, int z, int zb);
-
 __device__ __forceinline__ long long wrap_node(const GridDev &g, int x, int y, int z, int zb)
 {
     int p[3] = {x, y, z};
@@ -627,13 +626,13 @@ __device__ __forceinline__ long long wrap_node(const GridDev &g, int x, int y, i
     return ((long long)p[2] * g.n[1] + p[1]) * g.n[0] + p[0];
 }
 
-// One CTA of kPushThreads per SM: the shared region of a tile holds most of the SM's shared
-// memory, and 1024 threads at 64 registers (a few spills) hide more latency than 512 at 122.
+// The frozen species' kernel: move and deposit of particles whose momentum never changes (no gather, no
+// external field), crossing ones queued in shared memory.
 template <int ORDER, class Reg>
 __global__ void __launch_bounds__(kPushThreads, 1)
-k_push_frozen(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work, int *work_sparse, int *err, Reg reg)
+k_push_frozen(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, int *work, int *work_sparse, int *err, Reg reg)
 {
-    const ExtDev ext = ext_at_clock(ext0);
+    const ExtDev ext{};
     extern __shared__ float smem[];
     __shared__ int s_item, s_qn;
     __shared__ float s_js[3], s_jinv[3], s_dl[3];
@@ -698,7 +697,7 @@ k_push_frozen(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int
             }
         }
         __syncthreads();
-        // each lane takes gq consecutive particles (kGroup = 4 for a full item: half a cell of an
+        // each lane takes gq consecutive particles (4 for a full item: half a cell of an
         // 8-per-cell lattice, visited in octant order), and a warp's lanes sit NW * gq = 128
         // particles (16 cells of that lattice) apart, so at every iteration the 32 lanes sit on 32
         // different cells with the same stencil shift (bank-conflict-free shared accesses, see
@@ -888,7 +887,7 @@ inline bool default_region(const pic_ctx *c)
 }
 
 template <int ORDER, class Reg>
-cudaError_t launch_frozen_t(pic_ctx *c, int si, const ExtDev &ext, Reg reg, int R3)
+cudaError_t launch_frozen_t(pic_ctx *c, int si, Reg reg, int R3)
 {
     static KernelCache cache;
     const Species &s = c->sp[si];
@@ -898,22 +897,22 @@ cudaError_t launch_frozen_t(pic_ctx *c, int si, const ExtDev &ext, Reg reg, int 
     cudaError_t e = cache.blocks_per_sm((const void *)kern, c->dev.device, kPushThreads, smem, &per_sm);
     if (e != cudaSuccess) return e;
     kern<<<c->num_sms * per_sm, kPushThreads, smem, c->stream>>>(species_dev(c, s), grid_dev(c), tile_dev(c, s),
-                                                                  FieldsDev{c->E, c->B, c->J}, ext, c->work + si,
+                                                                  FieldsDev{c->E, c->B, c->J}, c->work + si,
                                                                   c->work + kMaxSpecies + si, c->err, reg);
     c->kernels++;
     return cudaGetLastError();
 }
 
 // Frozen species: the region spans the tile, its drift margin and the general deposit window.
-template <int ORDER> cudaError_t launch_frozen(pic_ctx *c, int si, const ExtDev &ext)
+template <int ORDER> cudaError_t launch_frozen(pic_ctx *c, int si)
 {
     if (default_region(c)) {
         constexpr int R = 8 + 2 * 1 + (ORDER == 1 ? 3 : 5);
-        return launch_frozen_t<ORDER>(c, si, ext, RegFix<R, R, R>{}, plane_pitch(R, R) * R);
+        return launch_frozen_t<ORDER>(c, si, RegFix<R, R, R>{}, plane_pitch(R, R) * R);
     }
     const TileDev t = tile_dev(c, c->sp[si]);
     const int P2 = plane_pitch(t.R[0], t.R[1]);
-    return launch_frozen_t<ORDER>(c, si, ext, RegDyn{t.R[0], t.R[1], P2, P2 * t.R[2]}, P2 * t.R[2]);
+    return launch_frozen_t<ORDER>(c, si, RegDyn{t.R[0], t.R[1], P2, P2 * t.R[2]}, P2 * t.R[2]);
 }
 
 }  // namespace push

@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(NT, MINB)
 k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work, int *work_sparse, int *err, Reg reg, int age)
 {
     using S = Shape<ORDER>;
-        const ExtDev ext = ext_at_clock(ext0);
+    const ExtDev ext = ext_at_clock(ext0);
     extern __shared__ __align__(16) float smem[];
     __shared__ int4 s_item;
     __shared__ float s_js[3], s_jinv[3], s_dl[3];
