@@ -37,8 +37,8 @@ __global__ void k_lattice_step(LatStepP p, int *err)
         PlaneRec r = p.planes[s];
         if (r.kz < 0) continue;
         // the move of a frozen particle with u = (0, 0, u_z); the roundings are spelt out, because a
-        // plasma's current is what is left of this one and the electrons' (the sum rounds twice, where
-        // the particle kernel's move rounds once)
+        // plasma's current is what is left of this one and the electrons' (the sum rounds twice, as a
+        // frozen particle's)
         const float ig = rsqrtf(1.f + p.uz * p.uz);
         const float d = __fmul_rn(__fmul_rn(p.uz, ig), p.dtdz);
         const float x1 = __fadd_rn(r.oz, d);

@@ -509,8 +509,10 @@ __device__ __forceinline__ void push_u(Acc &acc, const float o[3], const int c[3
 }
 
 // Move of one particle: v the velocity, d the displacement (cells), s the cell shift, o1 the new
-// offsets and c the new cell.  False when the particle left through a non-periodic face or its momentum is not finite
+// offsets and c the new cell.  ONCE has a bit for each dim whose new offset rounds once (the sum with the product v dt/d)
+// instead of twice (with the rounded displacement).  False when the particle left through a non-periodic face or its momentum is not finite
 // (it becomes a dummy).
+template <int ONCE>
 __device__ __forceinline__ bool move(const float o[3], int c[3], const float4 &mo, const GridDev &g, int *err, float d[3],
                                      int s[3], float o1[3], int zb, float v[3])
 {
@@ -520,13 +522,12 @@ __device__ __forceinline__ bool move(const float o[3], int c[3], const float4 &m
     bool alive = true;
 #pragma unroll
     for (int dd = 0; dd < 3; dd++) {
-        // the displacement of the push (cells), and the new offset with one rounding; both are spelt
-        // out, so that every path (and build) of the particle kernels moves a particle to the same
-        // place: a cold lattice's particles round alike, and a neutral plasma's current is a small
-        // difference of large ones
+        // the displacement of the push (cells) and the new offset; both are spelt out, so that every
+        // build moves a particle to the same place: a cold lattice's particles round alike, and a
+        // neutral plasma's current is a small difference of large ones
         v[dd] = __fmul_rn(u[dd], ig);
         d[dd] = __fmul_rn(v[dd], g.dt_over_d[dd]);
-        const float x1 = fmaf(v[dd], g.dt_over_d[dd], o[dd]);
+        const float x1 = (ONCE >> dd) & 1 ? fmaf(v[dd], g.dt_over_d[dd], o[dd]) : __fadd_rn(o[dd], d[dd]);
         s[dd] = (int)floorf(x1);
         o1[dd] = x1 - (float)s[dd];
         if (o1[dd] >= 1.f) { o1[dd] = 0.f; s[dd] += 1; }
@@ -543,13 +544,13 @@ __device__ __forceinline__ bool move(const float o[3], int c[3], const float4 &m
 }
 
 // Gather, external field, push (unless FROZEN) and move of one particle (see move).
-template <int ORDER, bool FROZEN, class Acc, int GATHER = 0>
+template <int ORDER, bool FROZEN, int ONCE, class Acc, int GATHER = 0>
 __device__ __forceinline__ bool push_move(Acc &acc, const float o[3], int c[3], float4 &mo,
                                           const SpeciesDev &sp, const GridDev &g, const ExtDev &ext,
                                           int *err, float d[3], int s[3], float o1[3], int zb, float v[3])
 {
     if (!FROZEN) push_u<ORDER, Acc, GATHER>(acc, o, c, mo, sp, ext);
-    return move(o, c, mo, g, err, d, s, o1, zb, v);
+    return move<ONCE>(o, c, mo, g, err, d, s, o1, zb, v);
 }
 
 // First node of the general deposit window, relative to the cell.
@@ -568,8 +569,11 @@ __device__ __forceinline__ bool stays_all(const float o[3], const float d[3], co
 }
 
 // Whole step of one particle's record on the global-memory path; dmax (may be NULL) takes the
-// largest displacement per component (float bits).
-template <int ORDER, bool FROZEN, int GATHER = 0>
+// largest displacement per component (float bits).  SPARSE: a record of a tile of a few.  Which dims
+// round once (offset and crossing length alike) is what every path always did, kept because two
+// programs' runs are compared to the last digits of a neutral plasma's fields: all of a mobile species'
+// but in sparse tiles, there z of TSC; none of a frozen species'.
+template <int ORDER, bool FROZEN, bool SPARSE, int GATHER = 0>
 __device__ __forceinline__ void step_record(float4 &P, float4 &mo, const SpeciesDev &sp, const GridDev &g, const FieldsDev &f,
                                             const ExtDev &ext, int *err, unsigned *dmax)
 {
@@ -580,12 +584,17 @@ __device__ __forceinline__ void step_record(float4 &P, float4 &mo, const Species
     GlobAcc<ORDER> acc(f, g, c, err, zb);
     float d[3], o1[3], v[3];
     int s[3];
-    if (push_move<ORDER, FROZEN, GlobAcc<ORDER>, GATHER>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb, v)) {
+    constexpr int ONCE = FROZEN ? 0 : (!SPARSE ? 7 : (ORDER == 2 ? 4 : 0));
+    if (push_move<ORDER, FROZEN, ONCE, GlobAcc<ORDER>, GATHER>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb, v)) {
         const float fac[3] = {sp.cf[0] * mo.w, sp.cf[1] * mo.w, sp.cf[2] * mo.w};
-        // (TSC, along z: from the product, see Shape)
-        const bool product = ORDER == 2 && !FROZEN;
-        const float vz[3] = {d[0], d[1], product ? v[2] : d[2]}, hz[3] = {1.f, 1.f, product ? g.dt_over_d[2] : 1.f};
-        deposit_general<ORDER>(acc, o, d, s, fac, vz, hz);
+        float h[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const bool product = (ONCE >> k) & 1;
+            v[k] = product ? v[k] : d[k];
+            h[k] = product ? g.dt_over_d[k] : 1.f;
+        }
+        deposit_general<ORDER>(acc, o, d, s, fac, v, h);
         P = make_float4(o1[0], o1[1], o1[2], __int_as_float(g.cc.pack(c[0], c[1], c[2])));
         if (dmax)
 #pragma unroll
@@ -595,14 +604,14 @@ __device__ __forceinline__ void step_record(float4 &P, float4 &mo, const Species
     }
 }
 
-template <int ORDER, bool FROZEN, int GATHER = 0>
+template <int ORDER, bool FROZEN, bool SPARSE, int GATHER = 0>
 __device__ __forceinline__ void step_global(const SpeciesDev &sp, const GridDev &g, const FieldsDev &f,
                                             const ExtDev &ext, int *err, int p)
 {
     float4 P = sp.pos[p];
     if (__float_as_int(P.w) < 0) return;
     float4 mo = sp.mom[p];
-    step_record<ORDER, FROZEN, GATHER>(P, mo, sp, g, f, ext, err, nullptr);
+    step_record<ORDER, FROZEN, SPARSE, GATHER>(P, mo, sp, g, f, ext, err, nullptr);
     if (!FROZEN) sp.mom[p] = mo;
     sp.pos[p] = P;
 }
@@ -658,7 +667,7 @@ k_push_frozen(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, int *work, int *
             const int p_begin = n_sorted + (item - n_tile_items) * chunk;
             const int p_end = min(p_begin + chunk, n_total);
             for (int p = p_begin + threadIdx.x; p < p_end; p += blockDim.x)
-                step_global<ORDER, true>(sp, g, f, ext, err, p);
+                step_global<ORDER, true, false>(sp, g, f, ext, err, p);
             continue;
         }
 
@@ -733,7 +742,7 @@ k_push_frozen(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, int *work, int *
                 fast = fast && r >= -t.M && r < t.T[dd] + t.M;
             }
             if (!fast) {
-                step_global<ORDER, true>(sp, g, f, ext, err, p);
+                step_global<ORDER, true, false>(sp, g, f, ext, err, p);
                 break;
             }
             float4 mo = sp.mom[p];
@@ -742,7 +751,7 @@ k_push_frozen(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, int *work, int *
             SmemAcc<Reg> acc{reg, nullptr, sJlo, sJhi, s_js, base};
             float d[3], o1[3], v[3];
             int s[3];
-            if (push_move<ORDER, true, SmemAcc<Reg>>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb, v)) {
+            if (push_move<ORDER, true, 0, SmemAcc<Reg>>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb, v)) {
                 const float fac[3] = {sp.cf[0] * mo.w, sp.cf[1] * mo.w, sp.cf[2] * mo.w};
 #pragma unroll
                 for (int k = 0; k < 3; k++) dm[k] = __float_as_uint(fabsf(d[k]));
@@ -834,7 +843,7 @@ k_push_frozen(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, int *work, int *
         if (it >= n_sparse) break;
         const int tile = t.sparse_tiles[it];
         const int pe = t.tile_start[tile + 1];
-        for (int p = t.tile_start[tile] + lane; p < pe; p += 32) step_global<ORDER, true>(sp, g, f, ext, err, p);
+        for (int p = t.tile_start[tile] + lane; p < pe; p += 32) step_global<ORDER, true, false>(sp, g, f, ext, err, p);
     }
 }
 

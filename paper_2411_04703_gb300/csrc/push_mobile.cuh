@@ -323,7 +323,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             int c[3] = {g.cc.i(cell), g.cc.j(cell), g.cc.k(cell)}, s[3];
             SmemAcc<Reg> acc{reg, sF, sJlo, sJhi, s_js, rel[2] * R2 + rel[1] * Rx + rel[0]};
             float d[3], o1[3], v[3];
-            if (!push_move<ORDER, false, SmemAcc<Reg>, GATHER>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb, v)) {
+            if (!push_move<ORDER, false, 7, SmemAcc<Reg>, GATHER>(acc, o, c, mo, sp, g, ext, err, d, s, o1, zb, v)) {
                 sp.pos[p].w = __int_as_float(-1);
                 continue;
             }
@@ -361,7 +361,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             float4 R = sp.pos[p], mo = sp.mom[p];
             int rel[3];
             if (!in_region(__float_as_int(R.w), rel)) {
-                step_record<ORDER, false, GATHER>(R, mo, sp, g, f, ext, err, dmax);
+                step_record<ORDER, false, false, GATHER>(R, mo, sp, g, f, ext, err, dmax);
                 sp.mom[p] = mo;
                 sp.pos[p] = R;
                 continue;
@@ -371,7 +371,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
             const int c0[3] = {c[0], c[1], c[2]};
             const float o[3] = {R.x, R.y, R.z};
             float d[3], o1[3], v[3], h[3] = {g.dt_over_d[0], g.dt_over_d[1], g.dt_over_d[2]};
-            if (!move(o, c, mo, g, err, d, s, o1, zb, v)) {   // (as in the first loop, which lists none that leaves)
+            if (!move<7>(o, c, mo, g, err, d, s, o1, zb, v)) {   // (as in the first loop, which lists none that leaves)
                 sp.pos[p].w = __int_as_float(-1);
                 continue;
             }
@@ -450,7 +450,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
     // appended particles not yet sorted, then sparse tiles (fewer than kSparse particles, a warp
     // each): staging and flushing a region would cost more than the global path of these few
     for (int p = n_sorted + blockIdx.x * NT + tid; p < n_total; p += gridDim.x * NT)
-        step_global<ORDER, false, GATHER>(sp, g, f, ext, err, p);
+        step_global<ORDER, false, false, GATHER>(sp, g, f, ext, err, p);
     const int n_sparse = sp.count[3];
     for (;;) {
         int it = 0;
@@ -459,7 +459,7 @@ k_push(SpeciesDev sp, GridDev g, TileDev t, FieldsDev f, ExtDev ext0, int *work,
         if (it >= n_sparse) break;
         const int tile = t.sparse_tiles[it];
         const int pe = t.tile_start[tile + 1];
-        for (int p = t.tile_start[tile] + lane; p < pe; p += 32) step_global<ORDER, false, GATHER>(sp, g, f, ext, err, p);
+        for (int p = t.tile_start[tile] + lane; p < pe; p += 32) step_global<ORDER, false, true, GATHER>(sp, g, f, ext, err, p);
     }
 }
 

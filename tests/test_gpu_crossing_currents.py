@@ -63,10 +63,10 @@ def _general(order, o, d, v, h):
     return st.astype(int), np.array(S0), np.array(DS)
 
 
-def _fixed(order, o, d, v, h, fs):
-    """Fixed-point contributions of one particle: window's first node [3, n], values [3][x][y][z][n]."""
+def _current(order, o, d, v, h, fs):
+    """Current of each particle: its window's first node [3, n], values [3][x][y][z][n]."""
     L = order + 2
-    w = [_general(order, o[k], d[k], v[k], h) for k in range(3)]
+    w = [_general(order, o[k], d[k], v[k], h[k]) for k in range(3)]
     A = [_fma(F(0.5) * np.ones_like(w[k][2]), w[k][2], w[k][1]) for k in range(3)]
     Q = [w[k][2] * F(1.0 / 12.0) for k in range(3)]
     P = []
@@ -80,8 +80,7 @@ def _fixed(order, o, d, v, h, fs):
     for k in range(3):
         a, b = (k + 1) % 3, (k + 2) % 3
         Y = _fma(A[a][:, None], A[b][None], (Q[a][:, None] * w[b][2][None]).astype(np.float64))
-        V = np.rint(P[k][:, None, None] * Y[None]).astype(np.int64)          # [k, a, b, n]
-        out.append(np.moveaxis(V, [0, 1, 2], [k, a, b]))
+        out.append(np.moveaxis(P[k][:, None, None] * Y[None], [0, 1, 2], [k, a, b]))   # from [k, a, b, n]
     return np.stack([w[k][0] for k in range(3)]), np.array(out)
 
 
@@ -120,13 +119,15 @@ def test_crossing_currents_bit_by_bit(order, copies, neutral):
     dlim = min(DT, F(4) * np.abs(d).max())
     js = F(2.0 ** (30 - np.frexp(F(1.1) * cf * wt * dlim)[1]))
     fs = [fac * js] * 3
-    st, near_form = _fixed(order, o, d, d, F(1), fs)
-    _, far_form = _fixed(order, o, d, v, DT, fs)
+    one = np.ones(3, F)
+    st, near_form = _current(order, o, d, d, one, fs)
+    _, far_form = _current(order, o, d, v, DT * one, fs)
+    near_form, far_form = (np.rint(f).astype(np.int64) for f in (near_form, far_form))
     sms = torch.cuda.get_device_properties(0).multi_processor_count * (1 if neutral else 2)
     chunk = CHUNK
     while chunk > CHUNK_MIN and n * copies // chunk < sms:
         chunk //= 2
-    want = np.zeros_like(near_form, dtype=F)
+    want = np.zeros(near_form.shape, F)
     for first in range(0, copies, chunk):
         length = min(chunk, copies - first)
         a = min(length, QUEUE) if neutral else length
@@ -172,3 +173,55 @@ def test_lattice_ions_move_bit_by_bit():
         z = z - np.floor(z)
     P = sim.get_particles(ions)
     assert np.array_equal(P["off"][np.argsort(P["id"]), 2], np.where(z >= 1, F(0), z))
+
+
+@pytest.mark.parametrize("order", [1, 2])
+@pytest.mark.parametrize("path", ["tile", "beyond its region", "sparse", "appended", "frozen", "frozen sparse"])
+def test_moves_and_global_currents_bit_by_bit(order, path):
+    # which dims of a move round once (offset and product v dt in one sum), and, on the global-memory path,
+    # the currents of single particles: their crossing lengths are from the product along the same dims
+    import torch
+    rng = np.random.default_rng(10 * order + len(path))
+    nt = GRID // TILE
+    cell = np.stack(np.meshgrid(*[np.arange(nt)] * 3, indexing="ij")).reshape(3, -1) * TILE + 4
+    n = cell.shape[1]
+    copies = 40 if path in ("tile", "beyond its region", "frozen") else 1
+    o = rng.random((3, n)).astype(F)
+    u = (rng.integers(-32, 33, (3, n)) / 8.0).astype(F)
+    wt = F(2.0 ** -10)
+    sim = api.Sim((GRID,) * 3, (1.0,) * 3, float(DT), 2.0, order=order, tuning={"tile": (8, 8, 8), "sort_every": 64, "margin": 0})
+    if path == "appended":
+        sim.step(1)                                       # the sort that the records then come after
+    sid = sim.load_species(-1.0, 1.0, np.repeat(cell + o.astype(np.float64), copies, axis=1),
+                           np.repeat(u.astype(np.float64), copies, axis=1), np.full(n * copies, float(wt)),
+                           frame=api.PIC_FRAME_BOOSTED, frozen=path.startswith("frozen"))
+    steps = 12 if path == "beyond its region" else 1
+    first = None
+    for _ in range(steps):
+        for c in range(6):
+            sim.set_field(c, np.zeros((GRID,) * 3, F))    # free flight
+        sim.step(1)
+        if first is None:
+            first = np.stack([sim.get_field(api.PIC_JX + k) for k in range(3)])
+    sim.sync()
+    P = sim.get_particles(sid)
+    got = P["off"][np.argsort(P["id"])][::copies].T
+
+    once = {"sparse": (order == 2) * np.array([0, 0, 1]), "frozen": np.zeros(3), "frozen sparse": np.zeros(3)}.get(path, np.ones(3))
+    ig = torch.rsqrt(torch.tensor(1.0 + (u.astype(np.float64) ** 2).sum(0), dtype=torch.float32, device="cuda")).cpu().numpy()
+    v = u * ig
+    d = v * DT
+    x = o
+    for _ in range(steps):
+        x = np.where(once[:, None] == 1, _fma(v, DT, x), x + d)
+        x = x - np.floor(x)
+        x = np.where(x >= 1, F(0), x)
+    assert np.array_equal(got, x)
+    if copies > 1:
+        return
+    prod = (once == 1)[:, None]
+    st, J = _current(order, o, d, np.where(prod, v, d), np.where(prod[:, 0], DT, F(1)), [F(1.0 / float(DT)) * wt] * 3)
+    near = F(0) if order == 1 else F(0.5)
+    for q in np.flatnonzero((np.floor(o + d + near) != np.floor(o + near)).any(0)):
+        x0, y0, z0 = cell[:, q] + st[:, q]
+        assert np.array_equal(first[:, z0:z0 + order + 2, y0:y0 + order + 2, x0:x0 + order + 2], np.swapaxes(J[..., q], 1, 3)), q
