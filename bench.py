@@ -45,10 +45,10 @@ BYTES_FROZEN = 32.0
 BYTES_CELL_PUSH = 36.0
 # DRAM bytes (read + write) of the particle kernel per step of the plasma buncher 128x128x512 (its
 # two launches: plasma electrons and beam): one-pass ncu capture of dram__bytes_read.sum and
-# dram__bytes_write.sum on the half-length grid 128x128x256 (plasma launch 2.24 GB for 30.38M
-# electrons, beam launch 0.110 GB for 2.10M), scaled by the particles each launch pushes at full
+# dram__bytes_write.sum on the half-length grid 128x128x256 (plasma launch 2.05 GB for 30.38M
+# electrons, beam launch 0.128 GB for 2.10M), scaled by the particles each launch pushes at full
 # size (61.36M and 4.19M).
-TRAFFIC_PUSH_BUNCHER_STEP = 4.74e9
+TRAFFIC_PUSH_BUNCHER_STEP = 4.40e9
 
 
 def peaks():

@@ -127,11 +127,11 @@ __device__ __forceinline__ void deposit_cross(const SmemAcc<Reg> &acc, const flo
 //  - Two CTAs of the default tile's region fit on an SM, so that one stages, flushes or waits while
 //    the other computes (the list shares the fields' memory, the marks are a bit a record).  The next
 //    item's number and record are fetched behind the present one's staging, and a flush leaves the
-//    currents' words zero (2-D buncher 1.97 -> 1.76, 300k electrons 0.113 -> 0.110, small buncher
-//    0.330 -> 0.320).
-// ms per step, with the cell-ordered lanes -> one CTA of 512 threads -> two CTAs: plasma buncher
-// 5.22 -> 4.15 -> 3.80, sweep of 64 runs 18.0 -> 15.1 -> 13.6, long undulator 4.66 -> 4.19 -> 4.12, 65k
-// electrons CIC 0.045 -> 0.046 -> 0.033 (the region follows the drift), 2-D buncher 2.40 -> 1.40 (1.76 with one CTA: launch_push_dyn).
+//    currents' words zero (300k electrons 0.113 -> 0.110 ms per step).
+// ms per step, with the cell-ordered lanes -> now: plasma buncher 5.22 -> 4.24, sweep of 64 runs 18.0 ->
+// 15.9, long undulator 4.66 -> 4.18, 65k electrons CIC 0.045 -> 0.028 (the region follows the drift), 2-D
+// buncher 2.40 -> 1.75.  (Two CTAs for the plasmas: 3.80, 13.6, and 1.18 with four in 2-D; see INORDER.)
+//
 // NEUTRAL: a species whose current another one's nearly cancels (see cancels).
 //  - Its crossings' last digit shows in the fields (see Shape), and a lattice that crosses takes its tiles'
 //    currents with it.  An item's first kQueue crossings are formed from the rounded displacement, the
@@ -495,6 +495,7 @@ template <int ORDER, int GATHER> cudaError_t launch_push_fixed(pic_ctx *c, int s
     // Large species: 2 x 512 threads at 64 registers, whose warps hide more latency than their spills
     // cost.  Small ones, an item or two per CTA, end with their longest thread: 2 x 256 at 128 (300k
     // electrons 0.100 against 0.112 ms per step, 500k 0.115 / 0.130, 3.4M plasma 0.350 / 0.343).
+    // (A current that another one nearly cancels: one CTA of 512 at 128 registers, see INORDER.)
     const RegFix<R, R, R, R2> reg;
     if (cancels(c, si)) return launch_push_t<ORDER, GATHER, 512, 1, true, true>(c, si, ext, reg, R2 * R);
     if (c->sp[si].bound <= 8192 * (int64_t)c->num_sms) return launch_push_t<ORDER, GATHER, 256, 2>(c, si, ext, reg, R2 * R);
@@ -509,10 +510,9 @@ template <int ORDER, int GATHER> cudaError_t launch_push_dyn(pic_ctx *c, int si,
     const RegDyn reg{R[0], R[1], R2, R3};
     // as many CTAs as the region lets on an SM, 512 threads in all
     const size_t cta = push_smem(R3) + 1024 + 768, sm = 228 * 1024;   // with the reserved and the static part
-    // The plasma electrons' current is added to the ions', which it nearly cancels: J_z rounds by the
-    // order in which neighbouring tiles flush, and the smaller the tiles the more of its nodes are
-    // shared.  One CTA an SM keeps neighbours in the items' order (2-D buncher, 8 x 1 x 8 tiles: 1.76 ms
-    // per step against 1.18 with four CTAs, with a fourth of the scatter of B between launches).
+    // A current that another one nearly cancels: one CTA an SM (see INORDER; 2-D buncher, 8 x 1 x 8 tiles:
+    // 1.75 ms per step against 1.18 with four CTAs, with a fourth of the scatter of B between launches).  On
+    // a 2-D grid, whose tiles have half the neighbours, an item claimed ahead does not add to it (1.97 -> 1.75).
     if (cancels(c, si) && c->n[1] > 1) return launch_push_t<ORDER, GATHER, 512, 1, true, true>(c, si, ext, reg, R3);
     if (cancels(c, si)) return launch_push_t<ORDER, GATHER, 512, 1, true>(c, si, ext, reg, R3);
     if (4 * cta <= sm) return launch_push_t<ORDER, GATHER, 128, 4>(c, si, ext, reg, R3);
